@@ -48,7 +48,8 @@ extern "C" {
                        (Section 4 pairs p = 4 with a fifth-order BSRK(8,5) whose coefficients
                        it does not print; es_set_tableau loads any explicit tableau) */
 
-#define ES_FP64 0  /* every operation in FP64 */
+#define ES_FP64 0  /* FP64, and 64-bit fixed point with per-element block exponents (58..63
+                      fractional bits) in the flux differencing where its error is no larger */
 #define ES_MIXED 1 /* FP32 fluxes/SATs/viscous terms; FP64 state, stage states,
                       entropy-variable increments, entropy sums and gamma solve */
 #define ES_FP64X 2 /* fluxes/SATs/viscous terms in float-float arithmetic on the FP32 pipe

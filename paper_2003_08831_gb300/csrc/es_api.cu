@@ -77,6 +77,35 @@ void lgl_tables(int p, double* x, double* w, double* D) {
   D[p * n + p] = p * (p + 1) / 4.0;
 }
 
+// The volume term's tables in fixed point (es_fx.cuh), from the nodes refined in long double
+// so that the tables carry more than the 53 bits of a double: Q_ij = omega_i D_ij =
+// c/(P_p(x_i) P_p(x_j) (x_i - x_j)), c = 2/(p(p+1)), antisymmetric by construction.
+void fx_tables(int p, int kw, long long* Q, long long* W) {
+  const int n = p + 1;
+  double xd[kMaxP1], wd[kMaxP1], Dd[kMaxP1 * kMaxP1];
+  lgl_tables(p, xd, wd, Dd);
+  long double x[kMaxP1], Pv[kMaxP1];
+  for (int i = 0; i < n; ++i) {
+    x[i] = xd[i];
+    for (int it = 0; it < 3; ++it) {
+      long double a = 1.0L, b = x[i];
+      for (int k = 1; k < p; ++k) {
+        const long double c = ((2 * k + 1) * x[i] * b - k * a) / (k + 1);
+        a = b;
+        b = c;
+      }
+      Pv[i] = b;
+      if (i > 0 && i < p) x[i] += (a - x[i] * b) / ((p + 1) * b);  // Newton on (1 - x^2) P_p'
+    }
+  }
+  const long double c = 2.0L / (p * (p + 1));
+  for (int i = 0; i < n; ++i) {
+    W[i] = llrintl(ldexpl(Pv[i] * Pv[i] / c, 63 - kw));
+    for (int j = 0; j < n; ++j)
+      Q[i * n + j] = i == j ? 0 : llrintl(ldexpl(c / (Pv[i] * Pv[j] * (x[i] - x[j])) / 4.0L, 65));
+  }
+}
+
 // Butcher tableaux (Section 4 names BSRK(4,3), RK(4,4) and, for p = 4, 5, BSRK(8,5)
 // and VRK(9,6), whose coefficients it does not print).
 struct Tableau {
@@ -209,6 +238,11 @@ void build_params(const es_config& C, Params* out) {
   P.Cd = FluxConst<double>::make(C.gamma_gas);
   P.Cf = FluxConst<float>::make(C.gamma_gas);
   P.Cff = FluxConst<ff>::make(C.gamma_gas);
+  while ((1 << P.fxKw) <= C.p * (C.p + 1) / 2) ++P.fxKw;
+  fx_tables(C.p, P.fxKw, P.fxQ, P.fxW);
+  while (P.fxKt < 62 && P.Cd.C1x >= std::ldexp(1.0, P.fxKt)) ++P.fxKt;
+  const long double gl = C.gamma_gas;
+  P.fxC = llrintl(ldexpl(2.0L * (gl + 1.0L) / (gl - 1.0L), 62 - P.fxKt));
   P.kappa_heat = C.mu > 0.0 ? C.mu * C.gamma_gas * C.R / ((C.gamma_gas - 1.0) * C.Pr) : 0.0;
   P.K = C.nx * C.ny * C.nz;
   P.diss = C.interface_diss;

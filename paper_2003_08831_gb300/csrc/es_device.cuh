@@ -65,6 +65,11 @@ struct Params {
   FluxConst<double> Cd;        // flux constants per precision (host-computed: no
   FluxConst<float> Cf;         // divisions or square roots in the kernels)
   FluxConst<ff> Cff;
+  // fixed-point tables of the FP64 volume term (es_fx.cuh)
+  long long fxQ[kMaxP1 * kMaxP1];  // omega_i D_ij / 4, 65 fractional bits
+  long long fxW[kMaxP1];           // 2^-fxKw / omega_i < 1, 63 fractional bits
+  long long fxC;                   // C1x 2^-fxKt < 1, 62 fractional bits
+  int fxKt, fxKw;
   int K;                       // elements in the group
   int diss;                    // Rusanov interface dissipation on/off
   int p1;                      // p + 1

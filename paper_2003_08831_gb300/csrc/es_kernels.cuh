@@ -1109,6 +1109,10 @@ constexpr auto vol_kernel() {
   else return k_volume<P1, TF, NS, EPB, THREADS, FACES>;
 }
 
+}  // namespace es
+#include "es_volume_fx.cuh"
+namespace es {
+
 // ---------------------------------------------------------------------------
 // Relaxation (one lane group per element, RelaxGroup).  Per node: X0 = d_rho/rho,
 // dv = (d_m - v d_rho)/rho, Y0 = (gam-1)(d_E - v.d_m + |v|^2 d_rho/2)/p,
@@ -1701,12 +1705,24 @@ void Launcher<P1, TF>::grad(const Params& P, const void* aux, void* fV, cudaStre
 }
 
 
+// the FP64 mode's Euler volume kernel (fixed-point flux differencing)
+template <int P1, int V>
+constexpr auto vol_fx_kernel() {
+  using C = VolFxCfg<P1, V>;
+  return k_volume_fx<P1, C::EPB, C::THREADS, C::REGS>;
+}
+
 template <int P1, typename TF, int V>
 cudaError_t volume_setup_v() {
   using C = VolCfg<P1, V>;
   const int smem = (int)VolSmem<P1, C::EPB, false>::template bytes<TF>();
-  cudaError_t e1 = cudaFuncSetAttribute(vol_kernel<P1, TF, false, C::EPB, C::THREADS>(),
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e1;
+  if constexpr (std::is_same<TF, double>::value)
+    e1 = cudaFuncSetAttribute(vol_fx_kernel<P1, V>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)VolFxSmem<P1, VolFxCfg<P1, V>::EPB>::bytes);
+  else
+    e1 = cudaFuncSetAttribute(vol_kernel<P1, TF, false, C::EPB, C::THREADS>(),
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   cudaError_t e2 = cudaFuncSetAttribute(vol_kernel<P1, TF, true, C::EPB, C::THREADS>(),
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return e1 != cudaSuccess ? e1 : e2;
@@ -1728,7 +1744,11 @@ void volume_v(const Params& P, const StageVol& sv, const TF* aux, const TF* F, c
   const size_t smem = VolSmem<P1, C::EPB, false>::template bytes<TF>();
   if (ns)
     vol_kernel<P1, TF, true, C::EPB, C::THREADS>()<<<grid, C::THREADS, smem, st>>>(P, sv, aux, F, FL, fV);
-  else
+  else if constexpr (std::is_same<TF, double>::value) {
+    using X = VolFxCfg<P1, V>;
+    vol_fx_kernel<P1, V>()<<<(P.K + X::EPB - 1) / X::EPB, X::THREADS, VolFxSmem<P1, X::EPB>::bytes, st>>>(P, sv, aux, F,
+                                                                                                     FL);
+  } else
     vol_kernel<P1, TF, false, C::EPB, C::THREADS>()<<<grid, C::THREADS, smem, st>>>(P, sv, aux, F, FL, fV);
 }
 

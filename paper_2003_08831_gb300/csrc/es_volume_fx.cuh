@@ -1,0 +1,371 @@
+// k_volume of the FP64 mode (Euler): flux differencing and face terms in 64-bit block fixed point
+// on the integer pipe (es_fx.cuh), FP64 for d and the element sums.
+//
+// Bound: the FP64 form spent 84 % of its time on the FP64 pipe (52 FP64 instructions per pair of
+// nodes, ~76 scheduler slots each).  A pair now takes about 230 integer and FP32 instructions, half
+// of them on the half-rate ALU pipe, which sets the time.  Taylor--Green 32^3 p = 3, one stage's
+// launch (mean of a step's three): 1089 us -> 258 us; p = 5, 11 x 9 x 13: 363 us -> 93 us.
+// Accuracy against long double (right-hand side, per variable): no larger error than FP64's in any
+// variable, half of it in the momentum; element sums equal to two digits.
+#pragma once
+#include "es_fx.cuh"
+
+namespace es {
+
+// High words of each element's extreme values: largest and smallest z1, z5, largest |z2..z4|.
+// kBad: a face flux or sum beyond the element's scales.
+enum { kMx1, kMn1, kMx5, kMn5, kMxV, kBad, kFxMeta };
+
+template <int P1, int EPB>
+struct VolFxSmem {
+  static constexpr int Np = P1 * P1 * P1;
+  static constexpr size_t red = 0;                                          // [2][EPB Np] doubles, over z
+  static constexpr size_t z = 0;                                            // [5][EPB Np] fx
+  static constexpr size_t acc = z + size_t(5) * EPB * Np * 8;               // [5][EPB Np] fx (slow elements: double)
+  static constexpr size_t pair = acc + size_t(5) * EPB * Np * 8;            // [EPB Np] z1, z5 as float pairs
+  static constexpr size_t w3 = pair + size_t(EPB) * Np * 16;                // [Np] omega_i omega_j omega_k
+  static constexpr size_t scale = w3 + size_t(Np) * 8;                      // [EPB] FxScale
+  static constexpr size_t meta = scale + EPB * sizeof(FxScale);             // [kFxMeta][EPB]
+  static constexpr size_t bytes = meta + size_t(kFxMeta) * EPB * sizeof(int);
+};
+
+// Position of node n in the tile's shared-memory planes.  P1 = 4: a permutation within the
+// element for which the 16 lines of any direction, at any position along the line, lie in 16
+// different 8-byte banks (plain order: 4-way conflicts along x1 and x2).
+template <int P1>
+__device__ __forceinline__ int fx_pos(int n) {
+  if (P1 != 4) return n;
+  const int k = n >> 4, j = (n >> 2) & 3, i = n & 3;
+  return (k << 4) | (((j + k) & 3) << 2) | ((i + k) & 3);
+}
+
+// largest biased exponent of the instance's metrics
+__device__ __forceinline__ int fx_metric_exponent(const InstGeom& G) {
+  return max(max(__double2hiint(G.metric[0]), __double2hiint(G.metric[1])), __double2hiint(G.metric[2])) >> 20;
+}
+
+// An LGL line of an element outside the fixed-point range, in FP64 with its face terms (the
+// arithmetic of volume_body), from the parameter vector in global memory; acc holds doubles
+template <int P1>
+__device__ __noinline__ void volume_line_fp64(const Params& P, const double* __restrict__ aux,
+                                              const double* __restrict__ F, const double* __restrict__ FL, int e,
+                                              int m, int ab, double met, double* acc, int stride) {
+  constexpr int P2 = P1 * P1, Np = P1 * P2;
+  const long long N = (long long)P.K * Np, g0 = (long long)e * Np;
+  const int a = ab % P1, b = ab / P1;
+  Zstate<double> z[P1];
+  double r[P1][5];
+  for (int i = 0; i < P1; ++i) {
+    const long long g = g0 + line_node<P1>(m, a, b, i);
+    for (int c = 0; c < kAux; ++c) z[i].z[c] = aux[c * N + g];
+    for (int v = 0; v < 5; ++v) r[i][v] = 0.0;
+  }
+  for (int i = 0; i < P1; ++i)
+    for (int j = i + 1; j < P1; ++j) {
+      double f[5];
+      ec_flux(z[i], z[j], m, P.Cd, f);
+      for (int v = 0; v < 5; ++v) {
+        r[i][v] = fma(P.D2[i * P1 + j], f[v], r[i][v]);
+        r[j][v] = fma(P.D2[j * P1 + i], f[v], r[j][v]);
+      }
+    }
+  const bool lo_b = at_boundary(P, e, m, 0);
+  const int em = lo_b ? e : neighbour(P, e, m, -1);
+  const double* Fm = lo_b ? FL : F;
+  for (int v = 0; v < 5; ++v) {
+    r[P1 - 1][v] = fma(P.inv_omega_end, F[((long long)(m * 5 + v) * P.K + e) * P2 + ab], r[P1 - 1][v]);
+    r[0][v] = fma(-P.inv_omega_end, Fm[((long long)(m * 5 + v) * P.K + em) * P2 + ab], r[0][v]);
+  }
+  for (int i = 0; i < P1; ++i) {
+    const int n = fx_pos<P1>(line_node<P1>(m, a, b, i));
+    for (int v = 0; v < 5; ++v) acc[v * stride + n] = fma(-met, r[i][v], m == 0 ? 0.0 : acc[v * stride + n]);
+  }
+}
+
+// One LGL line in fixed point: every unordered pair once, both nodes' sums in registers, the
+// face fluxes at both ends (f_hi, f_lo: plane stride fs), then each node's sum times
+// metric/omega_i into the element's accumulator.  Component order (z1, z_m, the other two, z5),
+// so that the flux needs no selects on the direction.  Returns false when a face flux (more than
+// a quarter, near: half, of the sums' range) or a sum does not fit the element's scales; the sums
+// of three directions then stay below 2^63.
+template <int P1, int TIER>
+__device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& sc, int m, int a, int b, fx wm,
+                                               const fx* __restrict__ z, const float4* __restrict__ zf,
+                                               const double* __restrict__ f_hi, const double* __restrict__ f_lo,
+                                               long long fs, fx* __restrict__ acc, int stride) {
+  const int c1 = m, c2 = m == 2 ? 0 : m + 1, c3 = m == 0 ? 2 : m - 1;
+  const int comp[5] = {0, (1 + c1) * stride, (1 + c2) * stride, (1 + c3) * stride, 4 * stride};
+  fx r[P1][5];
+#pragma unroll
+  for (int i = 0; i < P1; ++i)
+#pragma unroll
+    for (int c = 0; c < 5; ++c) r[i][c] = 0;
+  bool fits = true;
+  {
+    const int v[5] = {0, 1 + c1, 1 + c2, 1 + c3, 4};
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      const int emax = 1084 + fx_unit(sc, c == 0 ? 0 : (c == 4 ? 4 : 1));
+      const double hi = f_hi[v[c] * fs], lo = f_lo[v[c] * fs];
+      const int top = max(__double2hiint(hi) & 0x7fffffff, __double2hiint(lo) & 0x7fffffff) >> 20;
+      fits &= top <= emax - (TIER == kFxNear ? 1 : 2);
+      r[P1 - 1][c] = fx_from_double(hi, emax);
+      r[0][c] = -fx_from_double(lo, emax);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < P1 - 1; ++i) {
+    fx si[5];
+    const int ni = fx_pos<P1>(line_node<P1>(m, a, b, i));
+#pragma unroll
+    for (int c = 0; c < 5; ++c) si[c] = z[comp[c] + ni];
+    const float4 qi = zf[ni];
+    const FxPair fi[2] = {{qi.x, qi.y}, {qi.z, qi.w}};
+#pragma unroll
+    for (int j = i + 1; j < P1; ++j) {
+      fx sj[5], g[5];
+      const int nj = fx_pos<P1>(line_node<P1>(m, a, b, j));
+#pragma unroll
+      for (int c = 0; c < 5; ++c) sj[c] = z[comp[c] + nj];
+      const float4 qj = zf[nj];
+      const FxPair fj[2] = {{qj.x, qj.y}, {qj.z, qj.w}};
+      fx_flux<TIER>(si, fi, sj, fj, P.fxQ[i * P1 + j], sc, g);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        r[i][c] += g[c];
+        r[j][c] -= g[c];
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < P1; ++i) {
+    const int n = fx_pos<P1>(line_node<P1>(m, a, b, i));
+    const fx w = fx_mul63(P.fxW[i], wm);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      if (TIER == kFxFar) fits &= unsigned(fx_hi(r[i][c]) + 0x40000000) < 0x80000000u;  // |r| < 2^62
+      const fx val = fx_mul(r[i][c], w);
+      acc[comp[c] + n] = m == 0 ? val : acc[comp[c] + n] + val;
+    }
+  }
+  return fits;
+}
+
+// Tiles (elements per CTA, threads) and register bounds, measured on GB300 (one right-hand side,
+// 2 M nodes, us): the kernel waits on the latency of its dependent integer products, so few
+// registers pay until they spill into the sums.  p = 2: 199 at 16 x 160 and 96 registers (32 x 288:
+// 222); p = 3: 211 at 4 x 64 and 168 (128: 213, 96: 235; 8 x 128: 229); p = 4: 283 at 1 x 32 and
+// 128 (5 x 128: 286); p = 5: 328 at 2 x 96 and 168 (4 x 160: 353, 1 x 64: 409).
+template <int P1, int V> struct VolFxCfg;
+template <> struct VolFxCfg<3, 0> { static constexpr int EPB = 16, THREADS = 160, REGS = 100; };
+template <> struct VolFxCfg<3, 1> { static constexpr int EPB = 32, THREADS = 288, REGS = 100; };
+template <> struct VolFxCfg<3, 2> { static constexpr int EPB = 3, THREADS = 32, REGS = 100; };
+template <> struct VolFxCfg<4, 0> { static constexpr int EPB = 4, THREADS = 64, REGS = 168; };
+template <> struct VolFxCfg<4, 1> { static constexpr int EPB = 8, THREADS = 128, REGS = 128; };
+template <> struct VolFxCfg<4, 2> { static constexpr int EPB = 2, THREADS = 32, REGS = 128; };
+template <> struct VolFxCfg<5, 0> { static constexpr int EPB = 1, THREADS = 32, REGS = 128; };
+template <> struct VolFxCfg<5, 1> { static constexpr int EPB = 5, THREADS = 128, REGS = 128; };
+template <> struct VolFxCfg<5, 2> { static constexpr int EPB = 2, THREADS = 64, REGS = 128; };
+template <> struct VolFxCfg<6, 0> { static constexpr int EPB = 2, THREADS = 96, REGS = 168; };
+template <> struct VolFxCfg<6, 1> { static constexpr int EPB = 4, THREADS = 160, REGS = 128; };
+template <> struct VolFxCfg<6, 2> { static constexpr int EPB = 1, THREADS = 64, REGS = 168; };
+
+template <int P1, int EPB, int THREADS, int REGS>
+__global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx(const __grid_constant__ Params P,
+                                                       const __grid_constant__ StageVol sv,
+                                                       const double* __restrict__ aux, const double* __restrict__ F,
+                                                       const double* __restrict__ FL) {
+  using S = VolFxSmem<P1, EPB>;
+  constexpr int P2 = P1 * P1, Np = P1 * P2, ST = EPB * Np;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fx* z = reinterpret_cast<fx*>(smem_raw + S::z);
+  fx* acc = reinterpret_cast<fx*>(smem_raw + S::acc);
+  double* w3 = reinterpret_cast<double*>(smem_raw + S::w3);
+  FxScale* scale = reinterpret_cast<FxScale*>(smem_raw + S::scale);
+  int* meta = reinterpret_cast<int*>(smem_raw + S::meta);
+  float4* zf = reinterpret_cast<float4*>(smem_raw + S::pair);
+  double* red = reinterpret_cast<double*>(smem_raw + S::red);
+  const long long N = (long long)P.K * Np;
+  const int e0 = blockIdx.x * EPB;
+  const int nel = min(EPB, P.K - e0);
+  const int nn = nel * Np;
+
+  // the tile's parameter vector: each element's extreme values, then fixed point in their scales
+  {
+    constexpr int NT = (ST + THREADS - 1) / THREADS;
+    double ld[NT][kAux];
+    const double* __restrict__ src = aux + (long long)e0 * Np;
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+      const int t = threadIdx.x + i * THREADS;
+#pragma unroll
+      for (int c = 0; c < kAux; ++c)
+        if (t < nn) ld[i][c] = src[c * N + t];
+    }
+    for (int t = threadIdx.x; t < kFxMeta * EPB; t += THREADS) {
+      const int k = t / EPB;
+      meta[t] = k == kMn1 || k == kMn5 ? 0x7fffffff : 0;
+    }
+    for (int n = threadIdx.x; n < Np; n += THREADS)
+      w3[n] = P.omega[n % P1] * P.omega[(n / P1) % P1] * P.omega[n / P2];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+      const int t = threadIdx.x + i * THREADS;
+      if (t < nn) {
+        const int el = t / Np;
+        const int h1 = __double2hiint(ld[i][0]), h5 = __double2hiint(ld[i][4]);
+        const int hv = max(max(__double2hiint(ld[i][1]) & 0x7fffffff, __double2hiint(ld[i][2]) & 0x7fffffff),
+                           __double2hiint(ld[i][3]) & 0x7fffffff);
+        atomicMax(meta + kMx1 * EPB + el, h1);
+        atomicMin(meta + kMn1 * EPB + el, h1);
+        atomicMax(meta + kMx5 * EPB + el, h5);
+        atomicMin(meta + kMn5 * EPB + el, h5);
+        atomicMax(meta + kMxV * EPB + el, hv);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < nel) {
+      const int el = threadIdx.x;
+      scale[el] = fx_scale(meta[kMx1 * EPB + el], meta[kMn1 * EPB + el], meta[kMx5 * EPB + el],
+                           meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt);
+    }
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+      const int t = threadIdx.x + i * THREADS;
+      if (t < nn) {
+        const int el = t / Np;
+        const int ev = fx_block_exponent_v(meta[kMxV * EPB + el]);
+        fx* zt = z + el * Np + fx_pos<P1>(t - el * Np);
+        const fx z1 = fx_from_positive(ld[i][0], fx_block_exponent(meta[kMx1 * EPB + el]));
+        const fx z5 = fx_from_positive(ld[i][4], fx_block_exponent(meta[kMx5 * EPB + el]));
+        const FxPair p1 = fx_pair(z1), p5 = fx_pair(z5);
+        zf[zt - z] = make_float4(p1.h, p1.l, p5.h, p5.l);
+        zt[0] = z1;
+        zt[ST] = fx_from_double(ld[i][1], ev);
+        zt[2 * ST] = fx_from_double(ld[i][2], ev);
+        zt[3 * ST] = fx_from_double(ld[i][3], ev);
+        zt[4 * ST] = z5;
+      }
+    }
+  }
+  __syncthreads();
+
+#pragma unroll 1
+  for (int m = 0; m < 3; ++m) {
+    for (int l = threadIdx.x; l < nel * P2; l += THREADS) {
+      const int el = l / P2, ab = l % P2, e = e0 + el;
+      const FxScale& sc = scale[el];
+      if (sc.tier == kFxSlow) continue;
+      const InstGeom& G = geom_of(P, inst_of(P, e));
+      const int em = fx_metric_exponent(G);
+      const fx wm = fx_from_double(G.metric[m], em);
+      // this element's +x_m flux and the -x_m neighbour's (the boundary flux in FL)
+      const long long fs = (long long)P.K * P2;
+      const bool lo_b = at_boundary(P, e, m, 0);
+      const double* f_hi = F + m * 5 * fs + (long long)e * P2 + ab;
+      const double* f_lo = (lo_b ? FL : F) + m * 5 * fs + (long long)(lo_b ? e : neighbour(P, e, m, -1)) * P2 + ab;
+      const int a = ab % P1, b = ab / P1;
+      bool fits;
+      if (sc.tier == kFxNear)
+        fits = volume_line_fx<P1, kFxNear>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs,
+                                           acc + el * Np, ST);
+      else
+        fits = volume_line_fx<P1, kFxFar>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs,
+                                          acc + el * Np, ST);
+      if (!fits) meta[kBad * EPB + el] = 1;
+    }
+    __syncthreads();
+  }
+  // elements outside the fixed-point range, in FP64
+  const int my = threadIdx.x;
+  const bool slow = my < nel && (scale[my].tier == kFxSlow || meta[kBad * EPB + my]);
+  if (slow) scale[my].tier = kFxSlow;
+  if (__syncthreads_or(slow)) {
+#pragma unroll 1
+    for (int m = 0; m < 3; ++m) {
+      for (int l = threadIdx.x; l < nel * P2; l += THREADS) {
+        const int el = l / P2;
+        if (scale[el].tier != kFxSlow) continue;
+        volume_line_fp64<P1>(P, aux, F, FL, e0 + el, m, l % P2,
+                             geom_of(P, inst_of(P, e0 + el)).metric[m], reinterpret_cast<double*>(acc) + el * Np, ST);
+      }
+      __syncthreads();
+    }
+  }
+
+  // node phase: k_i = volume sums + face terms; d in the last stage; element sums (z is dead)
+  const bool wantE = sv.E != nullptr;
+  const bool wantA = sv.dw != nullptr;
+  for (int t = threadIdx.x; t < nn; t += THREADS) {
+    const long long g = (long long)e0 * Np + t;
+    const int el = t / Np, n = t % Np, e = e0 + el;
+    const InstGeom& G = geom_of(P, inst_of(P, e));
+    const FxScale& sc = scale[el];
+    double k[5];
+    const int at = el * Np + fx_pos<P1>(n);
+    if (sc.tier == kFxSlow) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) k[v] = reinterpret_cast<const double*>(acc)[v * ST + at];
+    } else {
+      const int em = fx_metric_exponent(G) - 1022 + P.fxKw + 2;  // metric: fraction of 2^(E + 1); fx_mul
+#pragma unroll
+      for (int v = 0; v < 5; ++v) k[v] = fx_to_double(-acc[v * ST + at], fx_unit(sc, v) + em);
+    }
+    if (sv.d_out) {
+      const double cs = sv.dcoef_self * G.dt;
+      double dv[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) dv[v] = cs * k[v];
+      for (int j = 0; j < sv.nd; ++j) {
+        const double cj = sv.dcoef[j] * G.dt;
+#pragma unroll
+        for (int v = 0; v < 5; ++v) dv[v] = fma(cj, static_cast<const double*>(sv.dk[j])[v * N + g], dv[v]);
+      }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sv.d_out[v * N + g] = dv[v];
+    } else {
+      double* ko = sv.kout64 ? sv.kout64 : static_cast<double*>(sv.kout);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) ko[v * N + g] = k[v];
+    }
+    if (wantE) {
+      Zstate<double> s;
+#pragma unroll
+      for (int c = 0; c < kAux; ++c) s.z[c] = aux[c * N + g];
+      double w[5];
+      z_to_w(s, P.Cd, w);
+      double sum = 0.0;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sum = fma(w[v], k[v], sum);
+      red[t] = w3[n] * sum;
+    }
+    if (wantA) {
+      double sum = 0.0;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sum = fma(sv.dw[v * N + g], k[v], sum);
+      red[ST + t] = w3[n] * sum;
+    }
+  }
+  const bool doA = sv.A != nullptr && (wantA || sv.A_init);
+  if (!wantE && !doA) return;
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int el = warp; el < nel; el += THREADS >> 5) {
+    const int e = e0 + el;
+    const InstGeom& G = geom_of(P, inst_of(P, e));
+    double sE = 0.0, sA = 0.0;
+    for (int n = lane; n < Np; n += 32) {
+      if (wantE) sE += red[el * Np + n];
+      if (wantA) sA += red[ST + el * Np + n];
+    }
+    if (wantE) sE = warp_sum(sE);
+    if (wantA) sA = warp_sum(sA);
+    if (lane == 0) {
+      if (wantE) sv.E[e] = G.J * sE;
+      if (doA) sv.A[e] = (sv.A_init ? 0.0 : sv.A[e]) + (wantA ? sv.A_scale * (G.J * G.dt) * sA : 0.0);
+    }
+  }
+}
+
+}  // namespace es
