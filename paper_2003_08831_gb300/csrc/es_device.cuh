@@ -69,7 +69,8 @@ struct Params {
   long long fxQ[kMaxP1 * kMaxP1];  // omega_i D_ij / 4, 65 fractional bits
   long long fxW[kMaxP1];           // 2^-fxKw / omega_i < 1, 63 fractional bits
   long long fxC;                   // C1x 2^-fxKt < 1, 62 fractional bits
-  int fxKt, fxKw;
+  long long fxG;                   // gam - 1 = fxG 2^(fxEg - 63), 2^62 <= fxG < 2^63
+  int fxKt, fxKw, fxEg;
   int K;                       // elements in the group
   int diss;                    // Rusanov interface dissipation on/off
   int p1;                      // p + 1

@@ -23,7 +23,9 @@
 #include <type_traits>
 
 #include "es_device.cuh"
+#include "es_face_fx.cuh"
 #include "es_launch.h"
+#include "es_prep_fx.cuh"
 
 namespace es {
 
@@ -369,6 +371,37 @@ __device__ __forceinline__ bool stage_z_ff(const Params& P, const ff uf[5], cons
 }
 
 // ---------------------------------------------------------------------------
+// FP64 forms of the stage preparation's pieces for states outside the fixed-point range
+// (es_prep_fx.cuh), out of line: they are rare and would cost the common path its registers.
+static __device__ __noinline__ bool param_vector_fp64(const double* y, double gam, double* z) {
+  const double rho = y[0];
+  const double ir = fast_rcp(rho);
+  const double v0 = y[1] * ir, v1 = y[2] * ir, v2 = y[3] * ir;
+  const double p = (gam - 1.0) * (y[4] - 0.5 * rho * (v0 * v0 + v1 * v1 + v2 * v2));
+  // z1 = sqrt(rho/p) = rho / sqrt(rho p), z5 = sqrt(rho p)
+  const double rs = rsqrt(rho * p);
+  const double z1 = rho * rs;
+  z[0] = z1;
+  z[1] = z1 * v0;
+  z[2] = z1 * v1;
+  z[3] = z1 * v2;
+  z[4] = rho * p * rs;
+  z[5] = p * rs;  // 1/z1 = sqrt(p/rho)
+  return rho > 0.0 && p > 0.0;
+}
+static __device__ __noinline__ void increment_fp64(const double* u, const double* e, double gam, double inv_gm1,
+                                                   double* dw) {
+  entropy_var_increment(u, e, gam, inv_gm1, dw);
+}
+// w(y) - w(u), e = y - u up to y's rounding; zy: y's fixed-point state if it has one
+__device__ __forceinline__ void stage_increment_w(const Params& P, const double u[5], const double e[5],
+                                                  const FxState* zy, double dw[5]) {
+  FxState zu;
+  if (zy && fx_state(u, P.fxG, P.fxEg, zu) && fx_increment(zu, *zy, P.fxC, P.fxKt, dw)) return;
+  increment_fp64(u, e, P.gam, P.Cd.inv_gm1, dw);
+}
+
+// ---------------------------------------------------------------------------
 // y = u (+ gamma d when the instance has a pending relaxed update and this is the
 // step's first stage) + dt sum_j a_ij k_j over the stages with a_ij != 0.
 // FP64 mode: everything in FP64.  Mixed mode with FP64 estimates (P.ff_est = 0):
@@ -402,8 +435,12 @@ __global__ void k_prep(Params P, StagePrep sp, TF* __restrict__ aux, int* __rest
 #pragma unroll
       for (int c = 0; c < 6; ++c) aux[c * N + g] = z[c];
       if (sp.dw) {
-        double dw[5];
-        entropy_var_increment(u, e, gam, P.Cd.inv_gm1, dw);
+        double y[5], dw[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) y[v] = u[v] + e[v];
+        FxState zy;
+        const bool ok = fx_state(y, P.fxG, P.fxEg, zy);
+        stage_increment_w(P, u, e, ok ? &zy : nullptr, dw);
 #pragma unroll
         for (int v = 0; v < 5; ++v) sp.dw[v * N + g] = dw[v];
       }
@@ -421,25 +458,18 @@ __global__ void k_prep(Params P, StagePrep sp, TF* __restrict__ aux, int* __rest
           for (int v = 0; v < 5; ++v) y[v] = fma(c, kj[v * N + g], y[v]);
         }
       }
-      const double rho = y[0];
-      const double ir = fast_rcp(rho);
-      const double v0 = y[1] * ir, v1 = y[2] * ir, v2 = y[3] * ir;
-      const double p = (gam - 1.0) * (y[4] - 0.5 * rho * (v0 * v0 + v1 * v1 + v2 * v2));
-      if (!(rho > 0.0) || !(p > 0.0)) atomicOr(status, kStatusNonphysical);
-      // z1 = sqrt(rho/p) = rho / sqrt(rho p), z5 = sqrt(rho p)
-      const double rs = rsqrt(rho * p);
-      const double z1 = rho * rs;
-      aux[0 * N + g] = z1;
-      aux[1 * N + g] = z1 * v0;
-      aux[2 * N + g] = z1 * v1;
-      aux[3 * N + g] = z1 * v2;
-      aux[4 * N + g] = rho * p * rs;
-      aux[5 * N + g] = p * rs;  // 1/z1 = sqrt(p/rho)
+      double z[6];
+      FxState zy;
+      const bool ok = fx_state(y, P.fxG, P.fxEg, zy);
+      if (ok) fx_state_planes(zy, z);
+      else if (!param_vector_fp64(y, gam, z)) atomicOr(status, kStatusNonphysical);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) aux[c * N + g] = z[c];
       if (sp.dw) {
         double e[5], dw[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) e[v] = y[v] - u[v];
-        entropy_var_increment(u, e, gam, P.Cd.inv_gm1, dw);
+        stage_increment_w(P, u, e, ok ? &zy : nullptr, dw);
 #pragma unroll
         for (int v = 0; v < 5; ++v) sp.dw[v * N + g] = dw[v];
       }
@@ -606,6 +636,28 @@ __device__ __forceinline__ Zstate<TF> bc_z(const double* v, TF& iz) {
   return z;
 }
 
+// the FP64 mode's interface flux outside the fixed-point range, out of line
+static __device__ __noinline__ void face_flux_fp64(const Zstate<double>& L, double izL, const Zstate<double>& R,
+                                                   double izR, int m, const FluxConst<double>& C, int diss,
+                                                   double* f) {
+  face_flux(L, izL, R, izR, m, C, diss, f);
+}
+// face_flux with k_face's constants: in FP64 mode through the fixed-point form (es_face_fx.cuh),
+// the matrix dissipation always in FP64
+template <typename TF>
+__device__ __forceinline__ void interface_flux(const Params& P, const FluxConst<TF>& C, const Zstate<TF>& L, TF izL,
+                                               const Zstate<TF>& R, TF izR, int m, TF f[5]) {
+  if constexpr (std::is_same<TF, double>::value) {
+    if (fx_face_flux(L.z, R.z, m, P.fxC, P.fxKt, C.sqrt_gam, P.diss, f)) {
+      if (P.diss == 2) matrix_dissipation(L, R, m, C, f);
+    } else {
+      face_flux_fp64(L, izL, R, izR, m, C, P.diss, f);
+    }
+  } else {
+    face_flux(L, izL, R, izR, m, C, P.diss, f);
+  }
+}
+
 // VPEN: with the diss^V penalty (a separate instantiation keeps the common path's
 // register count)
 template <int P1, typename TF, bool VPEN>
@@ -633,7 +685,7 @@ __global__ void k_face(Params P, const TF* __restrict__ aux, TF* __restrict__ F,
       izR = aux[5 * N + gR];
     }
     TF f[5];
-    face_flux(L, izL, R, izR, m, C, P.diss, f);
+    interface_flux(P, C, L, izL, R, izR, m, f);
     // diss^V penalty scale alpha (2/h_m)(1/omega_0)
     TF sig = TF(0);
     if constexpr (VPEN) {
@@ -648,7 +700,7 @@ __global__ void k_face(Params P, const TF* __restrict__ aux, TF* __restrict__ F,
       const long long g0 = (long long)e * Np + line_node<P1>(m, a, b, 0);
       const Zstate<TF> I = load_z<P1, TF>(aux, N, g0);
       const TF izI = aux[5 * N + g0];
-      face_flux(B, izB, I, izI, m, C, P.diss, f);
+      interface_flux(P, C, B, izB, I, izI, m, f);
       if constexpr (VPEN) visc_penalty(B, izB, I, izI, m, sig, P, f);
 #pragma unroll
       for (int v = 0; v < 5; ++v) FL[((long long)(m * 5 + v) * P.K + e) * P2 + ab] = f[v];
@@ -1662,14 +1714,24 @@ __global__ void k_estimate(Params P, const double* __restrict__ q, const double*
 
 // ---------------------------------------------------------------------------
 // launchers
+
+// Threads per block of the kernels that work node by node: blocks of 64 while blocks of 256 would
+// not give every SM one (152 SMs).
+inline int node_block(int& grid) {
+  if (grid > 152) return 256;
+  grid *= 4;
+  return 64;
+}
+
 template <typename TF, bool FP64>
 void prep_launch(const Params& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid) {
+  const int nb = node_block(grid);
   switch (sp.nprev) {
-    case 0: k_prep<TF, 0, FP64><<<grid, 256, 0, st>>>(P, sp, a, status); break;
-    case 1: k_prep<TF, 1, FP64><<<grid, 256, 0, st>>>(P, sp, a, status); break;
-    case 2: k_prep<TF, 2, FP64><<<grid, 256, 0, st>>>(P, sp, a, status); break;
-    case 3: k_prep<TF, 3, FP64><<<grid, 256, 0, st>>>(P, sp, a, status); break;
-    default: k_prep<TF, -1, FP64><<<grid, 256, 0, st>>>(P, sp, a, status); break;
+    case 0: k_prep<TF, 0, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
+    case 1: k_prep<TF, 1, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
+    case 2: k_prep<TF, 2, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
+    case 3: k_prep<TF, 3, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
+    default: k_prep<TF, -1, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
   }
 }
 
@@ -1689,10 +1751,11 @@ void Launcher<P1, TF>::prep(const Params& P, const StagePrep& sp, void* aux, int
 
 template <int P1, typename TF>
 void Launcher<P1, TF>::face(const Params& P, const void* aux, void* F, void* FL, cudaStream_t st, int grid) {
+  const int nb = node_block(grid);
   if (P.visc_pen > 0.0)
-    k_face<P1, TF, true><<<grid, 256, 0, st>>>(P, static_cast<const TF*>(aux), static_cast<TF*>(F), static_cast<TF*>(FL));
+    k_face<P1, TF, true><<<grid, nb, 0, st>>>(P, static_cast<const TF*>(aux), static_cast<TF*>(F), static_cast<TF*>(FL));
   else
-    k_face<P1, TF, false><<<grid, 256, 0, st>>>(P, static_cast<const TF*>(aux), static_cast<TF*>(F), static_cast<TF*>(FL));
+    k_face<P1, TF, false><<<grid, nb, 0, st>>>(P, static_cast<const TF*>(aux), static_cast<TF*>(F), static_cast<TF*>(FL));
 }
 
 template <int P1, typename TF>
