@@ -277,7 +277,7 @@ ES_HD fx fx_series_far(fx r) {
 struct FxScale {
   int tier;        // kFxSlow: outside the fixed-point range, FP64 flux
   int e1, e5, ev;  // largest biased exponents
-  int sv, sp;      // right shifts of the convective and the pressure part of the momentum flux
+  int sv, sp, se;  // right shifts of the convective and the pressure part of the momentum flux, of the energy flux
   int kt, ss;      // t < 2^kt; right shift of |S_v|^2
   fx C;            // C1x 2^-kt, 63 fractional bits
 };
@@ -291,13 +291,20 @@ ES_HD int fx_block_exponent_v(int mxv) {
   return e > 1007 ? e : 1007;
 }
 
+// Room in the momentum and energy sums beyond the element's own fluxes: none; kFxViscous: the energy
+// sum's unit follows the velocity scale only down to Mach ~1/16 (heat conduction does not vanish
+// with the velocity); kFxCoarse: face and viscous fluxes up to 2^6 times the pressure and the
+// enthalpy flux at sound speed (the second attempt of an element that did not fit).
+constexpr int kFxFine = 0, kFxViscous = 1, kFxCoarse = 2;
+
 // From the high words of the element's largest and smallest z1 and z5 and largest |z2..z4|.
 // Fast when z1 and z5 are positive and vary by less than a factor 1.5 (u <= 0.04 for every
 // pair; NaN, infinities and signs fall through the comparisons of the high words), their
 // exponents leave every product inside the double range, and |z_v| < 4 (Mach below ~3.4).  Gas at
 // rest (|z_v| < 2^-30) stays in FP64: there the volume sums have to cancel the face fluxes' bits
 // (what remains is all that an undisturbed element next to a discontinuity moves by).
-ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int ktg) {
+ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int ktg,
+                       int room = kFxFine) {
   FxScale s;
   s.e1 = fx_block_exponent(mx1);
   s.e5 = fx_block_exponent(mx5);
@@ -311,8 +318,10 @@ ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int k
   const bool near = (a1 - b1 + 1) * 100 <= a1 + b1 && (a5 - b5 + 1) * 100 <= a5 + b5;
   s.tier = !(ok && far) ? kFxSlow : (near ? kFxNear : kFxFar);
   const int Ev = s.ev - 1022;
-  s.sv = Ev < 0 ? -2 * Ev : 0;
-  s.sp = Ev > 0 ? 2 * Ev : 0;
+  const int c = room == kFxCoarse ? 6 : 0;
+  s.sv = (Ev < 0 ? -2 * Ev : 0) + c;
+  s.sp = (Ev > 0 ? 2 * Ev : 0) + c;
+  s.se = room == kFxFine ? 0 : (room == kFxCoarse ? (Ev < 0 ? -Ev : 0) + 6 : (Ev < -4 ? -Ev - 4 : 0));
   s.kt = (ktg > 2 * Ev + 3 ? ktg : 2 * Ev + 3) + 1;
   s.ss = s.kt - 2 - 2 * Ev;
   s.C = (C1 >> ((s.kt - 1 - ktg) & 63));
@@ -321,7 +330,7 @@ ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int k
 // exponents of the flux sums' units: 2 Q_ij times the flux is n 2^unit for mass, momentum and energy
 ES_HD int fx_unit(const FxScale& s, int v) {
   const int E1 = s.e1 - 1022, E5 = s.e5 - 1022, Ev = s.ev - 1022;
-  return v == 0 ? E5 + Ev - 59 : (v < 4 ? E5 - E1 + s.sp - 59 : E5 + Ev - 2 * E1 + s.kt - 60);
+  return v == 0 ? E5 + Ev - 59 : (v < 4 ? E5 - E1 + s.sp - 59 : E5 + Ev - 2 * E1 + s.kt - (s.tier == kFxNear ? 61 : 60) + s.se);
 }
 
 // Twice Q_ij = omega_i D_ij times the Ismail--Roe flux between two nodes, in units of 2^fx_unit
@@ -331,7 +340,7 @@ ES_HD int fx_unit(const FxScale& s, int v) {
 //   pq = Q S5/S1, M = g pq S_m, mass flux M S1, momentum M S_k (+ pq for k = m),
 //   energy u_m (g pq t + 2^(1-kt) pq), u_m = S_m/S1, t = C1x f1 + |S_v|^2/2 (scaled by 2^-kt).
 // Every factor Q multiplies once, so the pair enters both nodes' sums with opposite signs.
-// Bounds: 1/3 <= S1 < 1, so inv < 3, pq < 0.57, |u_m| < 3, t < 0.95.
+// Bounds: 1/3 <= S1 < 1 (near: 0.49), so inv < 3 (2.05), pq < 0.57 (0.39), |u_m| < 3, t < 0.95.
 template <int TIER>
 ES_HD void fx_flux(const fx a[5], const FxPair fa[2], const fx b[5], const FxPair fb[2], fx Q, const FxScale& c,
                    fx g[5]) {
@@ -356,7 +365,7 @@ ES_HD void fx_flux(const fx a[5], const FxPair fa[2], const fx b[5], const FxPai
   g[2] = fx_mul(Ms, Sa);
   g[3] = fx_mul(Ms, Sb);
   const fx y = fx_mul(pg, t) + (pq >> c.kt);                                           // 61
-  g[4] = fx_mul63(fx_mul(Sm, inv) * 4, y * 4);                                         // 61
+  g[4] = fx_mul63(fx_mul(Sm, inv) * 4, y * (TIER == kFxNear ? 8 : 4)) >> c.se;         // 62, far: 61
 }
 
 }  // namespace es

@@ -20,6 +20,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "es_device.cuh"
@@ -1715,6 +1716,9 @@ __global__ void k_estimate(Params P, const double* __restrict__ q, const double*
 // ---------------------------------------------------------------------------
 // launchers
 
+// Meshes that leave SMs idle: a tile of one element and all three directions takes 12 to 21 us up to
+// 512 elements where the larger tiles take 21 to 39 (p = 2, 3, 5); at 1000 elements they meet for p = 3.
+constexpr int kSmallMesh = 600;
 // Threads per block of the kernels that work node by node: blocks of 64 while blocks of 256 would
 // not give every SM one (152 SMs).
 inline int node_block(int& grid) {
@@ -1768,26 +1772,28 @@ void Launcher<P1, TF>::grad(const Params& P, const void* aux, void* fV, cudaStre
 }
 
 
-// the FP64 mode's Euler volume kernel (fixed-point flux differencing)
-template <int P1, int V>
+// the FP64 mode's volume kernel (fixed-point flux differencing)
+template <int P1, int V, bool NS>
 constexpr auto vol_fx_kernel() {
   using C = VolFxCfg<P1, V>;
-  return k_volume_fx<P1, C::EPB, C::THREADS, C::REGS>;
+  return k_volume_fx<P1, C::EPB, C::THREADS, C::REGS, NS, V == kVolFxSmall ? 3 : 1>;
 }
 
 template <int P1, typename TF, int V>
 cudaError_t volume_setup_v() {
-  using C = VolCfg<P1, V>;
-  const int smem = (int)VolSmem<P1, C::EPB, false>::template bytes<TF>();
-  cudaError_t e1;
-  if constexpr (std::is_same<TF, double>::value)
-    e1 = cudaFuncSetAttribute(vol_fx_kernel<P1, V>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)VolFxSmem<P1, VolFxCfg<P1, V>::EPB>::bytes);
-  else
+  cudaError_t e1, e2;
+  if constexpr (std::is_same<TF, double>::value) {
+    const int smem = (int)VolFxSmem<P1, VolFxCfg<P1, V>::EPB>::bytes;
+    e1 = cudaFuncSetAttribute(vol_fx_kernel<P1, V, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e2 = cudaFuncSetAttribute(vol_fx_kernel<P1, V, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  } else {
+    using C = VolCfg<P1, V>;
+    const int smem = (int)VolSmem<P1, C::EPB, false>::template bytes<TF>();
     e1 = cudaFuncSetAttribute(vol_kernel<P1, TF, false, C::EPB, C::THREADS>(),
                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaError_t e2 = cudaFuncSetAttribute(vol_kernel<P1, TF, true, C::EPB, C::THREADS>(),
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e2 = cudaFuncSetAttribute(vol_kernel<P1, TF, true, C::EPB, C::THREADS>(),
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  }
   return e1 != cudaSuccess ? e1 : e2;
 }
 
@@ -1796,23 +1802,24 @@ cudaError_t Launcher<P1, TF>::volume_setup() {
   cudaError_t e = volume_setup_v<P1, TF, 0>();
   if (e == cudaSuccess) e = volume_setup_v<P1, TF, 1>();
   if (e == cudaSuccess) e = volume_setup_v<P1, TF, 2>();
+  if constexpr (std::is_same<TF, double>::value)
+    if (e == cudaSuccess) e = volume_setup_v<P1, TF, kVolFxSmall>();
   return e;
 }
 
 template <int P1, typename TF, int V>
 void volume_v(const Params& P, const StageVol& sv, const TF* aux, const TF* F, const TF* FL, const TF* fV, bool ns,
               cudaStream_t st) {
-  using C = VolCfg<P1, V>;
-  const int grid = (P.K + C::EPB - 1) / C::EPB;
-  const size_t smem = VolSmem<P1, C::EPB, false>::template bytes<TF>();
-  if (ns)
-    vol_kernel<P1, TF, true, C::EPB, C::THREADS>()<<<grid, C::THREADS, smem, st>>>(P, sv, aux, F, FL, fV);
-  else if constexpr (std::is_same<TF, double>::value) {
-    using X = VolFxCfg<P1, V>;
-    vol_fx_kernel<P1, V>()<<<(P.K + X::EPB - 1) / X::EPB, X::THREADS, VolFxSmem<P1, X::EPB>::bytes, st>>>(P, sv, aux, F,
-                                                                                                     FL);
-  } else
-    vol_kernel<P1, TF, false, C::EPB, C::THREADS>()<<<grid, C::THREADS, smem, st>>>(P, sv, aux, F, FL, fV);
+  if constexpr (std::is_same<TF, double>::value) {
+    using C = VolFxCfg<P1, V>;
+    const auto k = ns ? vol_fx_kernel<P1, V, true>() : vol_fx_kernel<P1, V, false>();
+    k<<<(P.K + C::EPB - 1) / C::EPB, C::THREADS, VolFxSmem<P1, C::EPB>::bytes, st>>>(P, sv, aux, F, FL, fV);
+  } else {
+    using C = VolCfg<P1, V>;
+    const auto k = ns ? vol_kernel<P1, TF, true, C::EPB, C::THREADS>() : vol_kernel<P1, TF, false, C::EPB, C::THREADS>();
+    k<<<(P.K + C::EPB - 1) / C::EPB, C::THREADS, VolSmem<P1, C::EPB, false>::template bytes<TF>(), st>>>(P, sv, aux, F,
+                                                                                                    FL, fV);
+  }
 }
 
 template <int P1, typename TF>
@@ -1822,6 +1829,8 @@ void Launcher<P1, TF>::volume(const Params& P, const StageVol& sv, const void* a
   const TF* f = static_cast<const TF*>(F);
   const TF* fl = static_cast<const TF*>(FL);
   const TF* v = static_cast<const TF*>(fV);
+  if constexpr (std::is_same<TF, double>::value)
+    if (P.K <= kSmallMesh) return volume_v<P1, TF, kVolFxSmall>(P, sv, a, f, fl, v, ns, st);
   if (variant == 1) volume_v<P1, TF, 1>(P, sv, a, f, fl, v, ns, st);
   else if (variant == 2) volume_v<P1, TF, 2>(P, sv, a, f, fl, v, ns, st);
   else volume_v<P1, TF, 0>(P, sv, a, f, fl, v, ns, st);
@@ -1870,11 +1879,13 @@ void Launcher<P1, TF>::relax(const Params& P, const StageRelax& sr, cudaStream_t
   // the u_new entry point (es_relax_step), the FP64 mode and the mixed mode with FP64
   // estimates solve in FP64; 4 warps per block, RelaxGroup::EPW elements per warp
   const bool fp64 = sr.u_new || std::is_same<TF, double>::value || (std::is_same<TF, float>::value && !P.ff_est);
-  const int epb = 4 * (fp64 ? RelaxGroup<P1>::EPW : RelaxGroup<P1, true>::EPW);
-  const int need = (P.K + epb - 1) / epb;
-  const int g = grid < need ? grid : need;
-  if (fp64) k_relax<P1><<<g, 128, 0, st>>>(P, sr);
-  else k_relax_ff<P1><<<g, 128, 0, st>>>(P, sr);
+  // (one warp per block while four would leave SMs idle)
+  const int epw = fp64 ? RelaxGroup<P1>::EPW : RelaxGroup<P1, true>::EPW;
+  const int warps = P.K < 4 * epw * 152 ? 1 : 4;
+  const int need = (P.K + warps * epw - 1) / (warps * epw);
+  const int g = std::min(grid * 4 / warps, need);
+  if (fp64) k_relax<P1><<<g, 32 * warps, 0, st>>>(P, sr);
+  else k_relax_ff<P1><<<g, 32 * warps, 0, st>>>(P, sr);
 }
 
 template <int P1, typename TF>

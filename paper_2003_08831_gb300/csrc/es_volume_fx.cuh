@@ -1,5 +1,5 @@
-// k_volume of the FP64 mode (Euler): flux differencing and face terms in 64-bit block fixed point
-// on the integer pipe (es_fx.cuh), FP64 for d and the element sums.
+// k_volume of the FP64 mode: flux differencing, face terms and viscous divergence in 64-bit block
+// fixed point on the integer pipe (es_fx.cuh), FP64 for d and the element sums.
 //
 // Bound: the FP64 form spent 84 % of its time on the FP64 pipe (52 FP64 instructions per pair of
 // nodes, ~76 scheduler slots each).  A pair now takes about 230 integer and FP32 instructions, half
@@ -14,7 +14,8 @@ namespace es {
 
 // High words of each element's extreme values: largest and smallest z1, z5, largest |z2..z4|.
 // kBad: a face flux or sum beyond the element's scales.
-enum { kMx1, kMn1, kMx5, kMn5, kMxV, kBad, kFxMeta };
+// kRetry: the element is in its second attempt.
+enum { kMx1, kMn1, kMx5, kMn5, kMxV, kBad, kRetry, kFxMeta };
 
 template <int P1, int EPB>
 struct VolFxSmem {
@@ -46,10 +47,11 @@ __device__ __forceinline__ int fx_metric_exponent(const InstGeom& G) {
 
 // An LGL line of an element outside the fixed-point range, in FP64 with its face terms (the
 // arithmetic of volume_body), from the parameter vector in global memory; acc holds doubles
-template <int P1>
+template <int P1, bool NS>
 __device__ __noinline__ void volume_line_fp64(const Params& P, const double* __restrict__ aux,
-                                              const double* __restrict__ F, const double* __restrict__ FL, int e,
-                                              int m, int ab, double met, double* acc, int stride) {
+                                              const double* __restrict__ F, const double* __restrict__ FL,
+                                              const double* __restrict__ fV, int e, int m, int ab, double met,
+                                              double* acc, int stride) {
   constexpr int P2 = P1 * P1, Np = P1 * P2;
   const long long N = (long long)P.K * Np, g0 = (long long)e * Np;
   const int a = ab % P1, b = ab / P1;
@@ -76,6 +78,24 @@ __device__ __noinline__ void volume_line_fp64(const Params& P, const double* __r
     r[P1 - 1][v] = fma(P.inv_omega_end, F[((long long)(m * 5 + v) * P.K + e) * P2 + ab], r[P1 - 1][v]);
     r[0][v] = fma(-P.inv_omega_end, Fm[((long long)(m * 5 + v) * P.K + em) * P2 + ab], r[0][v]);
   }
+  if (NS) {
+    const int ep = neighbour(P, e, m, +1);
+    for (int c = 0; c < 4; ++c) {
+      const double* fc = fV + (long long)(m * 4 + c) * N;
+      double fl[P1];
+      for (int j = 0; j < P1; ++j) fl[j] = fc[g0 + line_node<P1>(m, a, b, j)];
+      const double f_next =
+          at_boundary(P, e, m, 1) ? fl[P1 - 1] : fc[(long long)ep * Np + line_node<P1>(m, a, b, 0)];
+      const double f_prev = lo_b ? fl[0] : fc[(long long)em * Np + line_node<P1>(m, a, b, P1 - 1)];
+      for (int i = 0; i < P1; ++i) {
+        double s = 0.0;
+        for (int j = 0; j < P1; ++j) s = fma(P.D[i * P1 + j], fl[j], s);
+        if (i == P1 - 1) s += 0.5 * P.inv_omega_end * (f_next - fl[P1 - 1]);
+        if (i == 0) s -= 0.5 * P.inv_omega_end * (f_prev - fl[0]);
+        r[i][1 + c] -= s;
+      }
+    }
+  }
   for (int i = 0; i < P1; ++i) {
     const int n = fx_pos<P1>(line_node<P1>(m, a, b, i));
     for (int v = 0; v < 5; ++v) acc[v * stride + n] = fma(-met, r[i][v], m == 0 ? 0.0 : acc[v * stride + n]);
@@ -83,16 +103,22 @@ __device__ __noinline__ void volume_line_fp64(const Params& P, const double* __r
 }
 
 // One LGL line in fixed point: every unordered pair once, both nodes' sums in registers, the
-// face fluxes at both ends (f_hi, f_lo: plane stride fs), then each node's sum times
-// metric/omega_i into the element's accumulator.  Component order (z1, z_m, the other two, z5),
-// so that the flux needs no selects on the direction.  Returns false when a face flux (more than
-// a quarter, near: half, of the sums' range) or a sum does not fit the element's scales; the sums
-// of three directions then stay below 2^63.
-template <int P1, int TIER>
+// face fluxes at both ends (f_hi, f_lo: plane stride fs), for Navier--Stokes the viscous
+// divergence, then each node's sum times metric/omega_i into the element's accumulator.  Component order (z1, z_m, the other two, z5),
+// so that the flux needs no selects on the direction.  Returns false when a face flux (2^60, near:
+// 2^61), a viscous flux (2^58, 2^59) or a sum (2^61: the weighted sums of three directions stay
+// below 2^63) does not fit the element's scales; with the bounds of fx_flux no sum passes 2^63
+// before it is checked.
+// Viscous part: omega_i (D f + lifting)_i = sum_{j != i} Q_ij f_j + f_next/2 (i = p) - f_prev/2
+// (i = 0), the diagonal of D cancelling the lifting's interior half (fv: planes of this direction,
+// plane stride N; v_hi, v_lo: nodes whose values stand for f_next and f_prev).
+template <int P1, int TIER, bool NS, int DIRS>
 __device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& sc, int m, int a, int b, fx wm,
                                                const fx* __restrict__ z, const float4* __restrict__ zf,
                                                const double* __restrict__ f_hi, const double* __restrict__ f_lo,
-                                               long long fs, fx* __restrict__ acc, int stride) {
+                                               long long fs, const double* __restrict__ fv, long long g0,
+                                               long long v_hi, long long v_lo, long long N, fx* __restrict__ acc,
+                                               int stride) {
   const int c1 = m, c2 = m == 2 ? 0 : m + 1, c3 = m == 0 ? 2 : m - 1;
   const int comp[5] = {0, (1 + c1) * stride, (1 + c2) * stride, (1 + c3) * stride, 4 * stride};
   fx r[P1][5];
@@ -111,6 +137,34 @@ __device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& s
       fits &= top <= emax - (TIER == kFxNear ? 1 : 2);
       r[P1 - 1][c] = fx_from_double(hi, emax);
       r[0][c] = -fx_from_double(lo, emax);
+    }
+    if constexpr (NS) {
+#pragma unroll
+      for (int c = 1; c < 5; ++c) {
+        const int emax = 1083 + fx_unit(sc, c == 4 ? 4 : 1);  // twice the value: Q carries a factor 1/4 and 65 bits
+        const double* f = fv + (long long)(c == 4 ? 3 : v[c] - 1) * N;
+        double fl[P1];
+#pragma unroll
+        for (int j = 0; j < P1; ++j) fl[j] = f[g0 + line_node<P1>(m, a, b, j)];
+        const double hi = f[v_hi], lo = f[v_lo];
+        int top = max(__double2hiint(hi) & 0x7fffffff, __double2hiint(lo) & 0x7fffffff);
+        fx n[P1];
+#pragma unroll
+        for (int j = 0; j < P1; ++j) {
+          top = max(top, __double2hiint(fl[j]) & 0x7fffffff);
+          n[j] = fx_from_double(fl[j], emax);
+        }
+        fits &= (top >> 20) <= emax - (TIER == kFxNear ? 2 : 3);
+        r[P1 - 1][c] -= fx_from_double(hi, emax) >> 2;
+        r[0][c] += fx_from_double(lo, emax) >> 2;
+#pragma unroll
+        for (int i = 0; i < P1; ++i)
+#pragma unroll
+          for (int j = i + 1; j < P1; ++j) {
+            r[i][c] -= fx_mul(P.fxQ[i * P1 + j], n[j]);
+            r[j][c] += fx_mul(P.fxQ[i * P1 + j], n[i]);
+          }
+      }
     }
   }
 #pragma unroll
@@ -137,18 +191,22 @@ __device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& s
       }
     }
   }
+  int over = 0;
 #pragma unroll
   for (int i = 0; i < P1; ++i) {
     const int n = fx_pos<P1>(line_node<P1>(m, a, b, i));
     const fx w = fx_mul63(P.fxW[i], wm);
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
-      if (TIER == kFxFar) fits &= unsigned(fx_hi(r[i][c]) + 0x40000000) < 0x80000000u;  // |r| < 2^62
-      const fx val = fx_mul(r[i][c], w);
-      acc[comp[c] + n] = m == 0 ? val : acc[comp[c] + n] + val;
+      over |= fx_hi(r[i][c]) + 0x20000000;  // bits 30, 31 set unless |r| < 2^61
+      const fx val = fx_mul63(r[i][c], w);
+      if constexpr (DIRS == 3)  // integer sums: any order gives the same bits
+        atomicAdd(reinterpret_cast<unsigned long long*>(acc) + comp[c] + n, (unsigned long long)val);
+      else
+        acc[comp[c] + n] = m == 0 ? val : acc[comp[c] + n] + val;
     }
   }
-  return fits;
+  return fits && !(over & 0xc0000000);
 }
 
 // Tiles (elements per CTA, threads) and register bounds, measured on GB300 (one right-hand side,
@@ -156,25 +214,34 @@ __device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& s
 // registers pay until they spill into the sums.  p = 2: 199 at 16 x 160 and 96 registers (32 x 288:
 // 222); p = 3: 211 at 4 x 64 and 168 (128: 213, 96: 235; 8 x 128: 229); p = 4: 283 at 1 x 32 and
 // 128 (5 x 128: 286); p = 5: 328 at 2 x 96 and 168 (4 x 160: 353, 1 x 64: 409).
+// Variant 3 is for meshes of few elements, whatever tile is asked for (the bits are the same): one
+// element per CTA and a thread for every line of its three directions.
+constexpr int kVolFxSmall = 3;
 template <int P1, int V> struct VolFxCfg;
 template <> struct VolFxCfg<3, 0> { static constexpr int EPB = 16, THREADS = 160, REGS = 100; };
 template <> struct VolFxCfg<3, 1> { static constexpr int EPB = 32, THREADS = 288, REGS = 100; };
 template <> struct VolFxCfg<3, 2> { static constexpr int EPB = 3, THREADS = 32, REGS = 100; };
+template <> struct VolFxCfg<3, kVolFxSmall> { static constexpr int EPB = 1, THREADS = 32, REGS = 168; };
 template <> struct VolFxCfg<4, 0> { static constexpr int EPB = 4, THREADS = 64, REGS = 168; };
 template <> struct VolFxCfg<4, 1> { static constexpr int EPB = 8, THREADS = 128, REGS = 128; };
 template <> struct VolFxCfg<4, 2> { static constexpr int EPB = 2, THREADS = 32, REGS = 128; };
-template <> struct VolFxCfg<5, 0> { static constexpr int EPB = 1, THREADS = 32, REGS = 128; };
-template <> struct VolFxCfg<5, 1> { static constexpr int EPB = 5, THREADS = 128, REGS = 128; };
-template <> struct VolFxCfg<5, 2> { static constexpr int EPB = 2, THREADS = 64, REGS = 128; };
+template <> struct VolFxCfg<4, kVolFxSmall> { static constexpr int EPB = 1, THREADS = 64, REGS = 168; };
+template <> struct VolFxCfg<5, 0> { static constexpr int EPB = 5, THREADS = 128, REGS = 168; };
+template <> struct VolFxCfg<5, 1> { static constexpr int EPB = 1, THREADS = 32, REGS = 168; };
+template <> struct VolFxCfg<5, 2> { static constexpr int EPB = 2, THREADS = 64, REGS = 168; };
+template <> struct VolFxCfg<5, kVolFxSmall> { static constexpr int EPB = 1, THREADS = 96, REGS = 168; };
 template <> struct VolFxCfg<6, 0> { static constexpr int EPB = 2, THREADS = 96, REGS = 168; };
 template <> struct VolFxCfg<6, 1> { static constexpr int EPB = 4, THREADS = 160, REGS = 128; };
 template <> struct VolFxCfg<6, 2> { static constexpr int EPB = 1, THREADS = 64, REGS = 168; };
+template <> struct VolFxCfg<6, kVolFxSmall> { static constexpr int EPB = 1, THREADS = 128, REGS = 168; };
 
-template <int P1, int EPB, int THREADS, int REGS>
+// DIRS: directions worked on together, 1 (in turn, by the same threads) or 3 (small meshes)
+template <int P1, int EPB, int THREADS, int REGS, bool NS, int DIRS = 1>
 __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx(const __grid_constant__ Params P,
                                                        const __grid_constant__ StageVol sv,
                                                        const double* __restrict__ aux, const double* __restrict__ F,
-                                                       const double* __restrict__ FL) {
+                                                       const double* __restrict__ FL,
+                                                       const double* __restrict__ fV) {
   using S = VolFxSmem<P1, EPB>;
   constexpr int P2 = P1 * P1, Np = P1 * P2, ST = EPB * Np;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -228,7 +295,7 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
     if (threadIdx.x < nel) {
       const int el = threadIdx.x;
       scale[el] = fx_scale(meta[kMx1 * EPB + el], meta[kMn1 * EPB + el], meta[kMx5 * EPB + el],
-                           meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt);
+                           meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt, NS ? kFxViscous : kFxFine);
     }
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
@@ -251,44 +318,71 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
   }
   __syncthreads();
 
+  // all three directions; elements whose fluxes did not fit their scales once more in coarser ones
+  const int my = threadIdx.x;
 #pragma unroll 1
-  for (int m = 0; m < 3; ++m) {
-    for (int l = threadIdx.x; l < nel * P2; l += THREADS) {
-      const int el = l / P2, ab = l % P2, e = e0 + el;
-      const FxScale& sc = scale[el];
-      if (sc.tier == kFxSlow) continue;
-      const InstGeom& G = geom_of(P, inst_of(P, e));
-      const int em = fx_metric_exponent(G);
-      const fx wm = fx_from_double(G.metric[m], em);
-      // this element's +x_m flux and the -x_m neighbour's (the boundary flux in FL)
-      const long long fs = (long long)P.K * P2;
-      const bool lo_b = at_boundary(P, e, m, 0);
-      const double* f_hi = F + m * 5 * fs + (long long)e * P2 + ab;
-      const double* f_lo = (lo_b ? FL : F) + m * 5 * fs + (long long)(lo_b ? e : neighbour(P, e, m, -1)) * P2 + ab;
-      const int a = ab % P1, b = ab / P1;
-      bool fits;
-      if (sc.tier == kFxNear)
-        fits = volume_line_fx<P1, kFxNear>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs,
-                                           acc + el * Np, ST);
-      else
-        fits = volume_line_fx<P1, kFxFar>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs,
-                                          acc + el * Np, ST);
-      if (!fits) meta[kBad * EPB + el] = 1;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    if constexpr (DIRS == 3) {
+      for (int t = threadIdx.x; t < 5 * ST; t += THREADS)
+        if (attempt == 0 || (t % ST < nn && meta[kRetry * EPB + t % ST / Np])) acc[t] = 0;
+      __syncthreads();
     }
-    __syncthreads();
+#pragma unroll 1
+    for (int m0 = 0; m0 < 3; m0 += DIRS) {
+      for (int l3 = threadIdx.x; l3 < DIRS * nel * P2; l3 += THREADS) {
+        const int m = DIRS == 3 ? l3 / (nel * P2) : m0;
+        const int l = DIRS == 3 ? l3 - m * (nel * P2) : l3;
+        const int el = l / P2, ab = l % P2, e = e0 + el;
+        const FxScale& sc = scale[el];
+        if (sc.tier == kFxSlow || (attempt && !(meta[kRetry * EPB + el]))) continue;
+        const InstGeom& G = geom_of(P, inst_of(P, e));
+        const int em = fx_metric_exponent(G);
+        const fx wm = fx_from_double(G.metric[m], em);
+        // this element's +x_m flux and the -x_m neighbour's (the boundary flux in FL)
+        const long long fs = (long long)P.K * P2;
+        const bool lo_b = at_boundary(P, e, m, 0);
+        const double* f_hi = F + m * 5 * fs + (long long)e * P2 + ab;
+        const double* f_lo = (lo_b ? FL : F) + m * 5 * fs + (long long)(lo_b ? e : neighbour(P, e, m, -1)) * P2 + ab;
+        const int a = ab % P1, b = ab / P1;
+        const long long g0 = (long long)e * Np;
+        long long v_hi = 0, v_lo = 0;
+        if constexpr (NS) {  // boundary faces take the interior viscous flux
+          v_hi = at_boundary(P, e, m, 1) ? g0 + line_node<P1>(m, a, b, P1 - 1)
+                                         : (long long)neighbour(P, e, m, +1) * Np + line_node<P1>(m, a, b, 0);
+          v_lo = lo_b ? g0 + line_node<P1>(m, a, b, 0)
+                      : (long long)neighbour(P, e, m, -1) * Np + line_node<P1>(m, a, b, P1 - 1);
+        }
+        const double* fv = NS ? fV + (long long)(m * 4) * N : nullptr;
+        bool fits;
+        if (sc.tier == kFxNear)
+          fits = volume_line_fx<P1, kFxNear, NS, DIRS>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs, fv, g0,
+                                                 v_hi, v_lo, N, acc + el * Np, ST);
+        else
+          fits = volume_line_fx<P1, kFxFar, NS, DIRS>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs, fv, g0,
+                                                v_hi, v_lo, N, acc + el * Np, ST);
+        if (!fits) meta[kBad * EPB + el] = 1;
+      }
+      __syncthreads();
+    }
+    const bool bad = my < nel && scale[my].tier != kFxSlow && meta[kBad * EPB + my];
+    if (attempt == 0 && bad) {
+      scale[my] = fx_scale(meta[kMx1 * EPB + my], meta[kMn1 * EPB + my], meta[kMx5 * EPB + my], meta[kMn5 * EPB + my],
+                           meta[kMxV * EPB + my], P.fxC, P.fxKt, kFxCoarse);
+      meta[kRetry * EPB + my] = 1;
+      meta[kBad * EPB + my] = 0;
+    }
+    if (attempt == 1 && bad) scale[my].tier = kFxSlow;
+    if (!__syncthreads_or(bad)) break;
   }
   // elements outside the fixed-point range, in FP64
-  const int my = threadIdx.x;
-  const bool slow = my < nel && (scale[my].tier == kFxSlow || meta[kBad * EPB + my]);
-  if (slow) scale[my].tier = kFxSlow;
-  if (__syncthreads_or(slow)) {
+  if (__syncthreads_or(my < nel && scale[my].tier == kFxSlow)) {
 #pragma unroll 1
     for (int m = 0; m < 3; ++m) {
       for (int l = threadIdx.x; l < nel * P2; l += THREADS) {
         const int el = l / P2;
         if (scale[el].tier != kFxSlow) continue;
-        volume_line_fp64<P1>(P, aux, F, FL, e0 + el, m, l % P2,
-                             geom_of(P, inst_of(P, e0 + el)).metric[m], reinterpret_cast<double*>(acc) + el * Np, ST);
+        volume_line_fp64<P1, NS>(P, aux, F, FL, fV, e0 + el, m, l % P2, geom_of(P, inst_of(P, e0 + el)).metric[m],
+                                 reinterpret_cast<double*>(acc) + el * Np, ST);
       }
       __syncthreads();
     }
@@ -308,7 +402,7 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
 #pragma unroll
       for (int v = 0; v < 5; ++v) k[v] = reinterpret_cast<const double*>(acc)[v * ST + at];
     } else {
-      const int em = fx_metric_exponent(G) - 1022 + P.fxKw + 2;  // metric: fraction of 2^(E + 1); fx_mul
+      const int em = fx_metric_exponent(G) - 1022 + P.fxKw + 1;  // metric: fraction of 2^(E + 1)
 #pragma unroll
       for (int v = 0; v < 5; ++v) k[v] = fx_to_double(-acc[v * ST + at], fx_unit(sc, v) + em);
     }
