@@ -27,6 +27,7 @@
 #include "es_face_fx.cuh"
 #include "es_launch.h"
 #include "es_prep_fx.cuh"
+#include "es_relax_fx.cuh"
 
 namespace es {
 
@@ -180,15 +181,13 @@ __device__ __forceinline__ void entropy_var_increment_ff(const ff u[5], const ff
 // Lanes per element in the relaxation kernels: a group of SUB lanes solves one element,
 // so for small Np two or four elements share a warp and the per-element scalar work
 // (reductions, bracket and Newton logic, executed by every lane of the group) is paid
-// once per 16 or 8 lanes instead of once per warp.  The FP64 solve keeps 16-lane groups
-// up to p = 4 (8 nodes per lane there; 4 % faster than whole warps).  The float-float
-// solve (FF) holds twice the registers per node value and is latency-bound: it takes
-// whole warps from Np > 32 on (measured: 1 % faster for p = 3, where the FP64 solve is
-// 1 % slower).
+// once per 16 or 8 lanes instead of once per warp.  The fixed-point solve holds about 24
+// registers per node: four nodes per lane up to p = 4.  The float-float solve (FF) takes whole
+// warps from Np > 32 on (measured: 1 % faster for p = 3).
 template <int P1, bool FF = false>
 struct RelaxGroup {
   static constexpr int Np = P1 * P1 * P1;
-  static constexpr int SUB = Np <= 32 ? 8 : ((Np <= 128 && !FF) ? 16 : 32);
+  static constexpr int SUB = Np <= 32 ? 8 : ((Np <= 64 && !FF) ? 16 : 32);
   static constexpr int R = (Np + SUB - 1) / SUB;  // nodes per lane
   static constexpr int EPW = 32 / SUB;            // elements per warp
   static __device__ __forceinline__ unsigned mask(int lane) {
@@ -1177,148 +1176,292 @@ namespace es {
 // Near the root the error after a step s is ~ s^2 r''/(2 r') ~ s^2/g, so a step
 // |s| <= root_rtol g (default 1e-8) leaves an error ~1e-16 g: the updated iterate is
 // returned without another evaluation.
+//
+// The FP64 form spent its time on the FP64 pipe (about 60 instructions per node, and 90 more per
+// Newton step: es_fx.cuh has their price).  Elements whose increments are below 1/16 are now solved
+// in fixed point (es_relax_fx.cuh), in one pass over the nodes; the others, and whatever does not
+// fit, take the FP64 form, out of line.
 template <int P1>
-__global__ void k_relax(Params P, StageRelax sr) {
+__device__ __noinline__ double relax_element_fp64(const Params& P, const StageRelax& sr, int e, int sl, unsigned gmask,
+                                                  double A) {
   using RG = RelaxGroup<P1>;
   constexpr int Np = RG::Np, R = RG::R, SUB = RG::SUB;
   const long long N = (long long)P.K * Np;
   const double gam = P.gam;
   const double inv_gm1 = P.Cd.inv_gm1;
   const float gamf = tf_from_double<float>(gam);
+  const double J = geom_of(P, inst_of(P, e)).J;
+  RelaxNode nd[R];
+  double a_part = 0.0, s_part = 0.0;
+  float b_part = 0.0f;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int n = sl + SUB * r;
+    nd[r].X0 = nd[r].Y0 = nd[r].V2 = nd[r].c = 0.0;
+    if (n < Np) {
+      const long long g = (long long)e * Np + n;
+      double u[5], d[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) u[v] = sr.u[v * N + g];
+      if (sr.u_new) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) d[v] = sr.u_new[v * N + g] - u[v];
+      } else {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) d[v] = sr.d_in[v * N + g];
+      }
+      // one division: 1/(rho Pr), Pr = rho p
+      const double rho = u[0];
+      const double m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
+      const double Pr = (gam - 1.0) * (rho * u[4] - 0.5 * m2);
+      const double inv = fast_rcp(rho * Pr);
+      const double ir = Pr * inv, ip = rho * rho * inv;
+      const double v0 = u[1] * ir, v1 = u[2] * ir, v2 = u[3] * ir;
+      const double v2s = m2 * ir * ir;
+      const double dv0 = (d[1] - v0 * d[0]) * ir, dv1 = (d[2] - v1 * d[0]) * ir, dv2 = (d[3] - v2 * d[0]) * ir;
+      const double Pn = mass_weight<P1>(P, J, n);
+      nd[r].X0 = d[0] * ir;
+      nd[r].Y0 = (gam - 1.0) * (d[4] - (v0 * d[1] + v1 * d[2] + v2 * d[3]) + 0.5 * v2s * d[0]) * ip;
+      nd[r].V2 = rho * (dv0 * dv0 + dv1 * dv1 + dv2 * dv2) * ip;
+      nd[r].c = Pn * rho;
+      const double XY = nd[r].X0 - nd[r].Y0;
+      a_part += 0.5 * nd[r].c * (nd[r].X0 * nd[r].X0 + XY * XY * inv_gm1 + nd[r].V2);
+      s_part += nd[r].c;
+      // the starting point's cubic term in FP32, from the node values rounded on the
+      // integer pipe (the FP64 pipe bounds this kernel)
+      const RelaxNodeF nf{ff(tf_from_double<float>(nd[r].X0), 0.0f), ff(tf_from_double<float>(nd[r].Y0), 0.0f),
+                          ff(tf_from_double<float>(nd[r].V2), 0.0f), ff(0.0f, 0.0f)};
+      b_part = __fmaf_rn(tf_from_double<float>(nd[r].c), relax_node_cubic_f(nf, gamf), b_part);
+    }
+  }
+  const double a = group_sum<SUB>(a_part, gmask);
+  const double ssum = group_sum<SUB>(s_part, gmask);
+  // the cubic coefficient only moves the starting point: an FP32 sum
+  const double bcub = group_sum_f<SUB>(b_part, gmask);
+  double gk = __longlong_as_double(0x7ff0000000000000LL);  // +inf: unconstrained
+  // delta_kappa = sqrt(2 a / sum c) > delta_floor, compared without the root and the division
+  if (2.0 * a > sr.delta_floor * sr.delta_floor * ssum) {
+    if (!(A < 0.0)) {
+      if (sl == 0) atomicOr(sr.status, kStatusNoRoot);
+    } else {
+      double lo = 0.0, hi = sr.gamma_max;
+      bool hi_known = false;
+      // start: root of the cubic model a g^2 + b g^3 + A g (one Newton step on
+      // a + b g + A/g from the quadratic model's root -A/a), off by O(delta^2)
+      double gcur = -A * fast_rcp(a);
+      const double den = a + 2.0 * bcub * gcur;
+      if (den > 0.0) gcur -= bcub * gcur * gcur * fast_rcp(den);
+      gcur = fmin(fmax(gcur, 1e-3), sr.gamma_max);
+      for (int it = 0; it < 100; ++it) {
+        double sr_ = 0.0, sd_ = 0.0;
+        bool ok = true;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          double D, dD;
+          if (nd[r].c != 0.0) {
+            if (relax_node_eval(nd[r], gcur, gam, inv_gm1, D, dD)) {
+              sr_ += nd[r].c * D;
+              sd_ += nd[r].c * dD;
+            } else {
+              ok = false;
+            }
+          }
+        }
+        const bool phys = __all_sync(gmask, ok);
+        const double rv = group_sum<SUB>(sr_, gmask) + gcur * A;
+        const double dv = group_sum<SUB>(sd_, gmask) + A;
+        if (!phys || rv > 0.0) {
+          hi = gcur;
+          hi_known = true;
+        } else {
+          lo = gcur;
+        }
+        if (phys && rv == 0.0) {
+          gk = gcur;
+          break;
+        }
+        const double step = rv * fast_rcp(dv);
+        const double newton = gcur - step;
+        // converged: a step this small cannot leave the bracket by more than rounding
+        if (phys && dv > 0.0 && fabs(step) <= sr.root_rtol * gcur) {
+          gk = fmin(fmax(newton, lo), hi);
+          break;
+        }
+        const bool nok = phys && dv > 0.0 && isfinite(newton) && newton > lo && newton < hi;
+        if (hi - lo <= 8.881784197001252e-16 * fmax(1.0, gcur)) {  // 4 * 2^-52
+          gk = lo;
+          break;
+        }
+        if (nok) gcur = newton;
+        else if (!hi_known) gcur = (gcur >= sr.gamma_max) ? sr.gamma_max : fmin(2.0 * gcur, sr.gamma_max);
+        else gcur = 0.5 * (lo + hi);
+        if (!hi_known && lo >= sr.gamma_max) {  // r(gamma_max) <= 0: capped
+          gk = sr.gamma_max;
+          break;
+        }
+      }
+    }
+  }
+  return gk;
+}
+
+template <int SUB>
+__device__ __forceinline__ fx group_sum_fx(fx v, unsigned mask) {
+#pragma unroll
+  for (int o = SUB / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  return v;
+}
+template <int SUB>
+__device__ __forceinline__ int group_max(int v, unsigned mask) {
+#pragma unroll
+  for (int o = SUB / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(mask, v, o));
+  return v;
+}
+
+// Fixed-point solve of the element whose nodes the group holds; false: to the FP64 form.
+// T, Tf: the group's rows in shared memory.
+template <int P1>
+__device__ __forceinline__ bool relax_element_fx(const Params& P, const StageRelax& sr,
+                                                 const FxRelaxNode (&nd)[RelaxGroup<P1>::R], const double* w8, int sl,
+                                                 unsigned gmask, double A, double J, fx* T, float* Tf, double& gk) {
+  using RG = RelaxGroup<P1>;
+  constexpr int Np = RG::Np, R = RG::R, SUB = RG::SUB;
+  int bits = kRelaxNone, er = kRelaxNone, nb[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    nb[r] = fx_relax_bits(nd[r]);
+    bits = max(bits, nb[r]);
+    er = max(er, nd[r].er);
+  }
+  bits = group_max<SUB>(bits, gmask);
+  er = group_max<SUB>(er, gmask);
+  const int E = bits + 2;
+  if (E < kRelaxMinE || E > kRelaxMaxE) return false;
+  FxRelaxTerm t[R];
+  fx cd[R];
+  int ex[R];
+  float est = 0.0f, cs = 0.0f;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int n = sl + SUB * r;
+    t[r] = fx_relax_term(nd[r], E, er, w8[n < Np ? n : 0]);
+    cd[r] = fx_relax_d2(nd[r], t[r], nb[r], E, P.fxG, P.fxEg, ex + r);
+    est += fx_relax_estimate(cd[r], ex[r]);
+    cs += fx_fraction(t[r].cn) * fx_pow2(t[r].ce + 64);
+  }
+  est = group_sum_f<SUB>(est, gmask);
+  cs = group_sum_f<SUB>(cs, gmask);
+  // delta_kappa > delta_floor, left to FP64 where FP32 cannot tell
+  const float lhs = 2.0f * est * fx_pow2(2 * E);
+  const float rhs = float(sr.delta_floor * sr.delta_floor * P.Cd.gm1) * cs;
+  if (!(est > 1e-30f) || !(fabsf(lhs - rhs) > 1e-3f * rhs)) return false;
+  gk = __longlong_as_double(0x7ff0000000000000LL);  // +inf: unconstrained
+  if (lhs < rhs) return true;
+  if (!(A < 0.0)) {
+    if (sl == 0) atomicOr(sr.status, kStatusNoRoot);
+    return true;
+  }
+  const int unit = fx_relax_unit(est), kl = fx_relax_last(E), kf = fx_relax_first_f(E);
+  const fx gp1 = fx_relax_gp1(P.fxG, P.fxEg);
+  FxRelaxSeries s[R];
+  fx a = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    a += fx_shift(cd[r], ex[r] + unit);
+    s[r] = fx_relax_series(t[r], unit);
+  }
+  a = group_sum_fx<SUB>(a, gmask);
+#pragma unroll 1
+  for (int k = 3; k < kf; ++k) {
+    fx sp = 0, sm = 0, sx = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) fx_relax_next(s[r], sp, sm, sx);
+    const fx c = group_sum_fx<SUB>(fx_relax_coefficient(k, sp, sm, sx, gp1), gmask);
+    if (sl == 0) {
+      T[k] = c;
+      Tf[k] = fx_fraction(c);
+    }
+  }
+  if (kf <= kl) {
+    FxRelaxSeriesF f[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) f[r] = fx_relax_series_f(s[r]);
+#pragma unroll 1
+    for (int k = kf; k <= kl; ++k) {
+      float sp = 0.0f, sm = 0.0f, sx = 0.0f;
+#pragma unroll
+      for (int r = 0; r < R; ++r) fx_relax_next_f(f[r], sp, sm, sx);
+      const float c = group_sum_f<SUB>(fx_relax_coefficient_f(k, sp, sm, sx, gp1), gmask);
+      if (sl == 0) Tf[k] = c;
+    }
+  }
+  __syncwarp(gmask);
+  const fx g = fx_relax_root(a, unit, E, er, kf, kl, T, Tf, A, J, P.fxG, P.fxEg);
+  __syncwarp(gmask);
+  gk = fx_to_double(g, -61);
+  return g != 0 && gk < sr.gamma_max;
+}
+
+// UNEW: the entry point that hands in u_new and d_eta
+template <int P1, bool UNEW>
+__global__ void __launch_bounds__(128, P1 == 6 ? 3 : 4) k_relax(const __grid_constant__ Params P, const __grid_constant__ StageRelax sr) {
+  using RG = RelaxGroup<P1>;
+  constexpr int Np = RG::Np, R = RG::R, SUB = RG::SUB;
+  __shared__ double w8[Np];
+  __shared__ fx T[4 * RG::EPW][kRelaxOrders + 1];
+  __shared__ float Tf[4 * RG::EPW][kRelaxOrders + 1];
+  for (int n = threadIdx.x; n < Np; n += blockDim.x) w8[n] = mass_weight<P1>(P, 0.125, n);
+  __syncthreads();
+  const long long N = (long long)P.K * Np;
   const int lane = threadIdx.x & 31;
-  const int sl = lane % SUB;                  // lane within the element's group
+  const int sl = lane % SUB;  // lane within the element's group
   const unsigned gmask = RG::mask(lane);
   const int warps_per_block = blockDim.x >> 5;
-  for (int e = (blockIdx.x * warps_per_block + (threadIdx.x >> 5)) * RG::EPW + lane / SUB; e < P.K;
-       e += gridDim.x * warps_per_block * RG::EPW) {
+  const int group = (threadIdx.x >> 5) * RG::EPW + lane / SUB;
+  for (int e = (blockIdx.x * warps_per_block) * RG::EPW + group; e < P.K; e += gridDim.x * warps_per_block * RG::EPW) {
     const int inst = inst_of(P, e);
     const double J = geom_of(P, inst).J;
-    RelaxNode nd[R];
-    double a_part = 0.0, s_part = 0.0, A_part = 0.0;
-    float b_part = 0.0f;
+    FxRelaxNode nd[R];
+    bool ok = P.fxEg >= -3 && P.fxEg <= 1;  // gam from 17/16 to 3
+    double A_part = 0.0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int n = sl + SUB * r;
-      nd[r].X0 = nd[r].Y0 = nd[r].V2 = nd[r].c = 0.0;
+      nd[r] = fx_relax_empty();
       if (n < Np) {
         const long long g = (long long)e * Np + n;
         double u[5], d[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) u[v] = sr.u[v * N + g];
-        if (sr.u_new) {
+        if constexpr (UNEW) {
 #pragma unroll
           for (int v = 0; v < 5; ++v) d[v] = sr.u_new[v * N + g] - u[v];
           if (sr.d_out) {
 #pragma unroll
             for (int v = 0; v < 5; ++v) sr.d_out[v * N + g] = d[v];
           }
+          // A = sum P w(u).d - d_eta with w = ((gam - s)/(gam-1) - beta|v|^2/2, beta v, -beta)
+          const double gam = P.gam, rho = u[0];
+          const double m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
+          const double Pr = (gam - 1.0) * (rho * u[4] - 0.5 * m2);
+          const double inv = fast_rcp(rho * Pr);
+          const double ir = Pr * inv, beta = rho * (rho * rho * inv);
+          const double p = Pr * ir;
+          const double sp = log(p) - gam * log(rho);
+          const double w0 = (gam - sp) * P.Cd.inv_gm1 - 0.5 * beta * (m2 * ir * ir);
+          A_part += mass_weight<P1>(P, J, n) *
+                    (w0 * d[0] + beta * (u[1] * ir * d[1] + u[2] * ir * d[2] + u[3] * ir * d[3]) - beta * d[4]);
         } else {
 #pragma unroll
           for (int v = 0; v < 5; ++v) d[v] = sr.d_in[v * N + g];
         }
-        // one division: 1/(rho Pr), Pr = rho p
-        const double rho = u[0];
-        const double m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
-        const double Pr = (gam - 1.0) * (rho * u[4] - 0.5 * m2);
-        const double inv = fast_rcp(rho * Pr);
-        const double ir = Pr * inv, ip = rho * rho * inv;
-        const double v0 = u[1] * ir, v1 = u[2] * ir, v2 = u[3] * ir;
-        const double v2s = m2 * ir * ir;
-        const double dv0 = (d[1] - v0 * d[0]) * ir, dv1 = (d[2] - v1 * d[0]) * ir, dv2 = (d[3] - v2 * d[0]) * ir;
-        const double Pn = mass_weight<P1>(P, J, n);
-        nd[r].X0 = d[0] * ir;
-        nd[r].Y0 = (gam - 1.0) * (d[4] - (v0 * d[1] + v1 * d[2] + v2 * d[3]) + 0.5 * v2s * d[0]) * ip;
-        nd[r].V2 = rho * (dv0 * dv0 + dv1 * dv1 + dv2 * dv2) * ip;
-        nd[r].c = Pn * rho;
-        const double XY = nd[r].X0 - nd[r].Y0;
-        a_part += 0.5 * nd[r].c * (nd[r].X0 * nd[r].X0 + XY * XY * inv_gm1 + nd[r].V2);
-        s_part += nd[r].c;
-        // the starting point's cubic term in FP32, from the node values rounded on the
-        // integer pipe (the FP64 pipe bounds this kernel)
-        const RelaxNodeF nf{ff(tf_from_double<float>(nd[r].X0), 0.0f), ff(tf_from_double<float>(nd[r].Y0), 0.0f),
-                            ff(tf_from_double<float>(nd[r].V2), 0.0f), ff(0.0f, 0.0f)};
-        b_part = __fmaf_rn(tf_from_double<float>(nd[r].c), relax_node_cubic_f(nf, gamf), b_part);
-        if (sr.u_new) {
-          // A = sum P w(u).d - d_eta with w = ((gam - s)/(gam-1) - beta|v|^2/2, beta v, -beta)
-          const double beta = rho * ip;
-          const double p = Pr * ir;
-          const double sp = log(p) - gam * log(rho);
-          const double w0 = (gam - sp) * inv_gm1 - 0.5 * beta * v2s;
-          A_part += Pn * (w0 * d[0] + beta * (v0 * d[1] + v1 * d[2] + v2 * d[3]) - beta * d[4]);
-        }
+        ok = fx_relax_node(u, d, nd[r]) && ok;
       }
     }
-    const double a = group_sum<SUB>(a_part, gmask);
-    const double ssum = group_sum<SUB>(s_part, gmask);
-    // the cubic coefficient only moves the starting point: an FP32 sum
-    const double bcub = group_sum_f<SUB>(b_part, gmask);
-    double A;
-    if (sr.u_new) A = group_sum<SUB>(A_part, gmask) - sr.deta[e];
-    else A = sr.A[e];
-    double gk = __longlong_as_double(0x7ff0000000000000LL);  // +inf: unconstrained
-    // delta_kappa = sqrt(2 a / sum c) > delta_floor, compared without the root and the division
-    if (2.0 * a > sr.delta_floor * sr.delta_floor * ssum) {
-      if (!(A < 0.0)) {
-        if (sl == 0) atomicOr(sr.status, kStatusNoRoot);
-      } else {
-        double lo = 0.0, hi = sr.gamma_max;
-        bool hi_known = false;
-        // start: root of the cubic model a g^2 + b g^3 + A g (one Newton step on
-        // a + b g + A/g from the quadratic model's root -A/a), off by O(delta^2)
-        double gcur = -A * fast_rcp(a);
-        const double den = a + 2.0 * bcub * gcur;
-        if (den > 0.0) gcur -= bcub * gcur * gcur * fast_rcp(den);
-        gcur = fmin(fmax(gcur, 1e-3), sr.gamma_max);
-        for (int it = 0; it < 100; ++it) {
-          double sr_ = 0.0, sd_ = 0.0;
-          bool ok = true;
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            double D, dD;
-            if (nd[r].c != 0.0) {
-              if (relax_node_eval(nd[r], gcur, gam, inv_gm1, D, dD)) {
-                sr_ += nd[r].c * D;
-                sd_ += nd[r].c * dD;
-              } else {
-                ok = false;
-              }
-            }
-          }
-          const bool phys = __all_sync(gmask, ok);
-          const double rv = group_sum<SUB>(sr_, gmask) + gcur * A;
-          const double dv = group_sum<SUB>(sd_, gmask) + A;
-          if (!phys || rv > 0.0) {
-            hi = gcur;
-            hi_known = true;
-          } else {
-            lo = gcur;
-          }
-          if (phys && rv == 0.0) {
-            gk = gcur;
-            break;
-          }
-          const double step = rv * fast_rcp(dv);
-          const double newton = gcur - step;
-          // converged: a step this small cannot leave the bracket by more than rounding
-          if (phys && dv > 0.0 && fabs(step) <= sr.root_rtol * gcur) {
-            gk = fmin(fmax(newton, lo), hi);
-            break;
-          }
-          const bool nok = phys && dv > 0.0 && isfinite(newton) && newton > lo && newton < hi;
-          if (hi - lo <= 8.881784197001252e-16 * fmax(1.0, gcur)) {  // 4 * 2^-52
-            gk = lo;
-            break;
-          }
-          if (nok) gcur = newton;
-          else if (!hi_known) gcur = (gcur >= sr.gamma_max) ? sr.gamma_max : fmin(2.0 * gcur, sr.gamma_max);
-          else gcur = 0.5 * (lo + hi);
-          if (!hi_known && lo >= sr.gamma_max) {  // r(gamma_max) <= 0: capped
-            gk = sr.gamma_max;
-            break;
-          }
-        }
-      }
-    }
+    const double A = UNEW ? group_sum<SUB>(A_part, gmask) - sr.deta[e] : sr.A[e];
+    double gk;
+    if (!__all_sync(gmask, ok) || !relax_element_fx<P1>(P, sr, nd, w8, sl, gmask, A, J, T[group], Tf[group], gk))
+      gk = relax_element_fp64<P1>(P, sr, e, sl, gmask, A);
     if (sl == 0) {
       sr.gamma_elem[e] = gk;
       atomic_min_positive(sr.gmin_bits + inst, gk);
@@ -1884,7 +2027,8 @@ void Launcher<P1, TF>::relax(const Params& P, const StageRelax& sr, cudaStream_t
   const int warps = P.K < 4 * epw * 152 ? 1 : 4;
   const int need = (P.K + warps * epw - 1) / (warps * epw);
   const int g = std::min(grid * 4 / warps, need);
-  if (fp64) k_relax<P1><<<g, 32 * warps, 0, st>>>(P, sr);
+  if (fp64 && sr.u_new) k_relax<P1, true><<<g, 32 * warps, 0, st>>>(P, sr);
+  else if (fp64) k_relax<P1, false><<<g, 32 * warps, 0, st>>>(P, sr);
   else k_relax_ff<P1><<<g, 32 * warps, 0, st>>>(P, sr);
 }
 
