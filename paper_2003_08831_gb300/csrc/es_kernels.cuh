@@ -1163,6 +1163,7 @@ constexpr auto vol_kernel() {
 
 }  // namespace es
 #include "es_volume_fx.cuh"
+#include "es_grad_fx.cuh"
 namespace es {
 
 // ---------------------------------------------------------------------------
@@ -1907,11 +1908,19 @@ void Launcher<P1, TF>::face(const Params& P, const void* aux, void* F, void* FL,
 
 template <int P1, typename TF>
 void Launcher<P1, TF>::grad(const Params& P, const void* aux, void* fV, cudaStream_t st, int) {
-  using C = VolCfg<P1, 0>;
-  const int grid = (P.K + C::EPB - 1) / C::EPB;
-  const size_t smem = size_t(4) * C::EPB * P1 * P1 * P1 * sizeof(TF);
-  k_grad<P1, TF, C::EPB, C::THREADS><<<grid, C::THREADS, smem, st>>>(P, static_cast<const TF*>(aux),
-                                                                      static_cast<TF*>(fV));
+  if constexpr (std::is_same<TF, double>::value) {
+    using C = GradFxCfg<P1>;
+    const int grid = (P.K + C::EPB - 1) / C::EPB;
+    const size_t smem = size_t(4) * C::EPB * (P1 * P1 * P1 + 6 * P1 * P1) * sizeof(fx);
+    k_grad_fx<P1, C::EPB, C::THREADS>
+        <<<grid, C::THREADS, smem, st>>>(P, static_cast<const double*>(aux), static_cast<double*>(fV));
+  } else {
+    using C = VolCfg<P1, 0>;
+    const int grid = (P.K + C::EPB - 1) / C::EPB;
+    const size_t smem = size_t(4) * C::EPB * P1 * P1 * P1 * sizeof(TF);
+    k_grad<P1, TF, C::EPB, C::THREADS>
+        <<<grid, C::THREADS, smem, st>>>(P, static_cast<const TF*>(aux), static_cast<TF*>(fV));
+  }
 }
 
 
