@@ -1355,9 +1355,10 @@ __device__ __forceinline__ bool relax_element_fx(const Params& P, const StageRel
   // delta_kappa > delta_floor, left to FP64 where FP32 cannot tell
   const float lhs = 2.0f * est * fx_pow2(2 * E);
   const float rhs = float(sr.delta_floor * sr.delta_floor * P.Cd.gm1) * cs;
-  if (!(est > 1e-30f) || !(fabsf(lhs - rhs) > 1e-3f * rhs)) return false;
+  if (!(est > 1e-30f)) return false;
   gk = __longlong_as_double(0x7ff0000000000000LL);  // +inf: unconstrained
-  if (lhs < rhs) return true;
+  if (lhs < 0.999f * rhs) return true;               // (an infinite floor too: relaxation switched off)
+  if (!(lhs > 1.001f * rhs)) return false;
   if (!(A < 0.0)) {
     if (sl == 0) atomicOr(sr.status, kStatusNoRoot);
     return true;
