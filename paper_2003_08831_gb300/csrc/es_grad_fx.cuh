@@ -88,11 +88,11 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * 128))
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx* ws = reinterpret_cast<fx*>(smem_raw);  // [4][ST] interior, [4][SF] outer states of the faces
   fx* wf = ws + 4 * ST;
-  __shared__ unsigned meta[kGradMeta][EPB];
+  __shared__ int meta[kGradMeta][EPB];
   __shared__ fx sQ[P1 * P1];
   const long long N = (long long)P.K * Np;
   const int e0 = blockIdx.x * EPB, nel = min(EPB, P.K - e0), nn = nel * Np, nf = nel * Nf;
-  for (int t = threadIdx.x; t < kGradMeta * EPB; t += THREADS) meta[t / EPB][t % EPB] = t / EPB == kGMn1 ? 0xffffffffu : 0u;
+  for (int t = threadIdx.x; t < kGradMeta * EPB; t += THREADS) meta[t / EPB][t % EPB] = t / EPB == kGMn1 ? 0x7fffffff : 0;
   for (int t = threadIdx.x; t < P1 * P1; t += THREADS) {
     const int i = t / P1, j = t % P1;
     sQ[t] = i < j ? P.fxQ[i * P1 + j] : (i > j ? -P.fxQ[j * P1 + i] : 0);
@@ -115,20 +115,26 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * 128))
 #pragma unroll
     for (int c = 0; c < 4; ++c) z[c] = aux[c * N + (long long)e0 * Np + t];
   };
+  // (the high word of a negative or NaN z1 counts as beyond every exponent allowed)
   const auto extremes = [&](int el, const double z[4]) {
-    const unsigned h1 = __double2hiint(z[0]);  // (negative values: above every exponent allowed)
-    atomicMax(&meta[kGMx1][el], h1);
-    atomicMin(&meta[kGMn1][el], h1);
-    atomicMax(&meta[kGMxV][el], unsigned(max(max(__double2hiint(z[1]) & 0x7fffffff, __double2hiint(z[2]) & 0x7fffffff),
-                                             __double2hiint(z[3]) & 0x7fffffff)));
+    const int h1 = __double2hiint(z[0]), hp = h1 < 0 ? 0x7fffffff : h1;
+    const bool one = warp_uniform(el);
+    fx_smem_max(&meta[kGMx1][el], hp, one);
+    fx_smem_min(&meta[kGMn1][el], hp, one);
+    fx_smem_max(&meta[kGMxV][el],
+                max(max(__double2hiint(z[1]) & 0x7fffffff, __double2hiint(z[2]) & 0x7fffffff),
+                    __double2hiint(z[3]) & 0x7fffffff), one);
   };
   __syncthreads();
   double z[4];
-  for (int t = threadIdx.x; t < nn; t += THREADS) {
+  // (threads beyond the tile repeat its last node)
+  for (int t0 = 0; t0 < nn; t0 += THREADS) {
+    const int t = min(t0 + int(threadIdx.x), nn - 1);
     inner(t, z);
     extremes(t / Np, z);
   }
-  for (int t = threadIdx.x; t < nf; t += THREADS) {
+  for (int t0 = 0; t0 < nf; t0 += THREADS) {
+    const int t = min(t0 + int(threadIdx.x), nf - 1);
     outer(t, z);
     extremes(t / Nf, z);
   }
@@ -162,7 +168,7 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * 128))
   for (int t = threadIdx.x; t < nn; t += THREADS) {
     const int el = t / Np, n = t - el * Np, e = e0 + el;
     const InstGeom& G = geom_of(P, inst_of(P, e));
-    const unsigned mx1 = meta[kGMx1][el], mn1 = meta[kGMn1][el], mxv = meta[kGMxV][el];
+    const int mx1 = meta[kGMx1][el], mn1 = meta[kGMn1][el], mxv = meta[kGMxV][el];
     const int em = fx_metric_exponent(G);
     // z1 within a factor of two or so; exponents in +-100; NaN and signs fail the comparisons
     if (!constants || (mx1 >> 20) > 1121 || (mn1 >> 20) < 923 || (mx1 >> 20) - (mn1 >> 20) > 1 || (mxv >> 20) > 1121 ||

@@ -40,6 +40,30 @@ __device__ __forceinline__ int fx_pos(int n) {
   return (k << 4) | (((j + k) & 3) << 2) | ((i + k) & 3);
 }
 
+// Extremes per element in shared memory, one value of every lane (all lanes of the warp present): one
+// atomic for a warp within one element, else one per lane (which are taken one by one where they
+// meet at an address).  Taylor--Green 32^3 p = 3: k_volume_fx 265 -> 254 us per launch.
+__device__ __forceinline__ void fx_smem_max(int* at, int v, bool one) {
+  if (one) {
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicMax(at, v);
+  } else {
+    atomicMax(at, v);
+  }
+}
+__device__ __forceinline__ void fx_smem_min(int* at, int v, bool one) {
+  if (one) {
+    v = __reduce_min_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicMin(at, v);
+  } else {
+    atomicMin(at, v);
+  }
+}
+// whether all lanes of the warp hold the same value
+__device__ __forceinline__ bool warp_uniform(int v) {
+  return __all_sync(0xffffffffu, v == __shfl_sync(0xffffffffu, v, 0));
+}
+
 // largest biased exponent of the instance's metrics
 __device__ __forceinline__ int fx_metric_exponent(const InstGeom& G) {
   return max(max(__double2hiint(G.metric[0]), __double2hiint(G.metric[1])), __double2hiint(G.metric[2])) >> 20;
@@ -167,6 +191,9 @@ __device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& s
       }
     }
   }
+  // the element is done again in other scales, or in FP64: no pair of this line is formed (viscous
+  // shock p = 3 25^3, where a band of elements needs the second attempt: 744 -> 693 us per launch)
+  if (!fits) return false;
 #pragma unroll
   for (int i = 0; i < P1 - 1; ++i) {
     fx si[5];
@@ -206,7 +233,7 @@ __device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& s
         acc[comp[c] + n] = m == 0 ? val : acc[comp[c] + n] + val;
     }
   }
-  return fits && !(over & 0xc0000000);
+  return !(over & 0xc0000000);
 }
 
 // Tiles (elements per CTA, threads) and register bounds, measured on GB300 (one right-hand side,
@@ -267,7 +294,7 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
       const int t = threadIdx.x + i * THREADS;
 #pragma unroll
       for (int c = 0; c < kAux; ++c)
-        if (t < nn) ld[i][c] = src[c * N + t];
+        ld[i][c] = src[c * N + min(t, nn - 1)];
     }
     for (int t = threadIdx.x; t < kFxMeta * EPB; t += THREADS) {
       const int k = t / EPB;
@@ -278,18 +305,17 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-      const int t = threadIdx.x + i * THREADS;
-      if (t < nn) {
-        const int el = t / Np;
-        const int h1 = __double2hiint(ld[i][0]), h5 = __double2hiint(ld[i][4]);
-        const int hv = max(max(__double2hiint(ld[i][1]) & 0x7fffffff, __double2hiint(ld[i][2]) & 0x7fffffff),
-                           __double2hiint(ld[i][3]) & 0x7fffffff);
-        atomicMax(meta + kMx1 * EPB + el, h1);
-        atomicMin(meta + kMn1 * EPB + el, h1);
-        atomicMax(meta + kMx5 * EPB + el, h5);
-        atomicMin(meta + kMn5 * EPB + el, h5);
-        atomicMax(meta + kMxV * EPB + el, hv);
-      }
+      // (threads beyond the tile repeat its last node)
+      const int el = min(int(threadIdx.x) + i * THREADS, nn - 1) / Np;
+      const int h1 = __double2hiint(ld[i][0]), h5 = __double2hiint(ld[i][4]);
+      const int hv = max(max(__double2hiint(ld[i][1]) & 0x7fffffff, __double2hiint(ld[i][2]) & 0x7fffffff),
+                         __double2hiint(ld[i][3]) & 0x7fffffff);
+      const bool one = warp_uniform(el);
+      fx_smem_max(meta + kMx1 * EPB + el, h1, one);
+      fx_smem_min(meta + kMn1 * EPB + el, h1, one);
+      fx_smem_max(meta + kMx5 * EPB + el, h5, one);
+      fx_smem_min(meta + kMn5 * EPB + el, h5, one);
+      fx_smem_max(meta + kMxV * EPB + el, hv, one);
     }
     __syncthreads();
     if (threadIdx.x < nel) {
@@ -334,7 +360,8 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
         const int l = DIRS == 3 ? l3 - m * (nel * P2) : l3;
         const int el = l / P2, ab = l % P2, e = e0 + el;
         const FxScale& sc = scale[el];
-        if (sc.tier == kFxSlow || (attempt && !(meta[kRetry * EPB + el]))) continue;
+        if (sc.tier == kFxSlow || (attempt && !meta[kRetry * EPB + el])) continue;
+        if (DIRS == 1 && m && meta[kBad * EPB + el]) continue;  // (set in an earlier direction)
         const InstGeom& G = geom_of(P, inst_of(P, e));
         const int em = fx_metric_exponent(G);
         const fx wm = fx_from_double(G.metric[m], em);
