@@ -290,14 +290,6 @@ void ff_split_host(double d, float out[2]) {
 // A group: instances sharing the LGL degree and the physics, stored as one SoA
 // over the group's elements.  The single-instance context is a group of one;
 // a batch is one group per degree.
-// Dirichlet-penalty boundary data of a context (host copy; passed to k_bc_eval by value)
-struct BcSpec {
-  int kind[3];           // ES_BC_* per direction
-  double q[3][2][5];     // ES_BC_STATE: exterior states (left, right)
-  double vs[3][6];       // ES_BC_VISCOUS_SHOCK: V_f, alpha, H, speed, x_lo, x_hi
-  double gam;
-};
-
 struct Group {
   es_config cfg;  // physics (and, for a context, the mesh)
   int P1 = 0, Np = 0, K = 0, ninst = 0;
@@ -648,77 +640,6 @@ int group_init(Group& g, const es_config* insts, int n, int stages, bool own_sta
   return rc;
 }
 
-// Exterior values of the Dirichlet-penalty boundaries at time *t + t_off: one warp per
-// (direction, side).  ES_BC_VISCOUS_SHOCK evaluates the Section 4.1.2 profile: V in
-// (V_f, 1) solves x - speed t = (alpha/2) [log((1-V)(V-V_f)) + (1+V_f)/(1-V_f)
-// log((1-V)/(V-V_f))] (to the last bit), u = V, rho = 1/V, p from the constant
-// total enthalpy H, lab velocity u + speed along the direction.
-//
-// The bracket is cut into 33 parts per round, one interior point per lane, so that eleven rounds
-// reach the last bit of a double: an evaluation (two logarithms) is a chain of ~90 dependent FP64
-// operations, 3 us for a warp, and bisection by one thread needed 55 and more of them (502 us a
-// launch, four launches of an RK4 step; now 25 us).
-__global__ void k_bc_eval(BcSpec spec, const double* t, double t_off, double* out) {
-  const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (i >= 6) return;
-  const int m = i / 2, side = i % 2;
-  if (spec.kind[m] == ES_BC_PERIODIC) return;
-  const double g = spec.gam;
-  double q[5];
-  if (spec.kind[m] == ES_BC_STATE) {
-    for (int v = 0; v < 5; ++v) q[v] = spec.q[m][side][v];
-  } else {
-    const double vf = spec.vs[m][0], alpha = spec.vs[m][1], H = spec.vs[m][2], speed = spec.vs[m][3];
-    const double time = (t ? t[0] : 0.0) + t_off;
-    const double xi = spec.vs[m][4 + side] - speed * time;
-    const double c = (1.0 + vf) / (1.0 - vf);
-    // x(V) decreases; 2 (x(V) - xi)/alpha = (1 + c) log(1 - V) + (1 - c) log(V - V_f) - 2 xi/alpha
-    const double rhs = 2.0 * xi / alpha;
-    double lo = vf, hi = 1.0;
-    for (int it = 0; it < 40; ++it) {
-      const double mid = fma(hi - lo, (lane + 1) * (1.0 / 33.0), lo);
-      const bool inside = mid > lo && mid < hi;
-      const bool below = inside ? (1.0 + c) * log(1.0 - mid) + (1.0 - c) * log(mid - vf) > rhs : mid <= lo;
-      const unsigned above = ~__ballot_sync(0xffffffffu, below);  // lanes right of the root
-      const int first = above ? __ffs(above) - 1 : 32;
-      const double l = __shfl_sync(0xffffffffu, mid, first ? first - 1 : 0);
-      const double h = __shfl_sync(0xffffffffu, mid, first < 32 ? first : 31);
-      const double nlo = first ? fmax(l, lo) : lo, nhi = first < 32 ? fmin(h, hi) : hi;
-      if (nlo == lo && nhi == hi) break;  // neighbouring doubles
-      lo = nlo;
-      hi = nhi;
-    }
-    const double u = 0.5 * (lo + hi);
-    const double rho = 1.0 / u;
-    const double p = (g - 1.0) / g * rho * (H - 0.5 * u * u);
-    const double ul = u + speed;
-    for (int v = 0; v < 5; ++v) q[v] = 0.0;
-    q[0] = rho;
-    q[1 + m] = rho * ul;
-    q[4] = p / (g - 1.0) + 0.5 * rho * ul * ul;
-  }
-  if (lane) return;
-  const double rho = q[0];
-  const double v0 = q[1] / rho, v1 = q[2] / rho, v2 = q[3] / rho;
-  const double p = (g - 1.0) * (q[4] - 0.5 * rho * (v0 * v0 + v1 * v1 + v2 * v2));
-  const double z1 = sqrt(rho / p);
-  double* o = out + i * kBcVals;
-  o[0] = z1;
-  o[1] = z1 * v0;
-  o[2] = z1 * v1;
-  o[3] = z1 * v2;
-  o[4] = sqrt(rho * p);
-  o[5] = sqrt(p / rho);
-  o[6] = rho * v0 / p;
-  o[7] = rho * v1 / p;
-  o[8] = rho * v2 / p;
-  o[9] = -rho / p;
-}
-
-void launch_bc_eval(const BcSpec& spec, const double* t, double t_off, double* out, cudaStream_t st) {
-  k_bc_eval<<<1, 192, 0, st>>>(spec, t, t_off, out);
-}
-
 int grid_for(const Engine& e, long long n, int block) { return grid_for_sms(e.sm_count, n, block); }
 
 // One stage's right-hand side into kout or d (+ element sums), on state u (+ pending
@@ -736,12 +657,11 @@ int run_stage(Engine& E, Group& g, const StagePrep& sp, const StageVol& sv, cuda
       return last_launch_error();
     });
   }
-  if (g.any_bc) {  // exterior states at this stage's time t + c_i dt
-    timed(E, ES_KERNEL_OTHER, st, [&] { launch_bc_eval(g.bc, t_dev ? t_dev : g.t, t_off, g.bcz, st); });
-  }
+  const BcEval bc{g.bc, t_dev ? t_dev : g.t, t_off, g.bcz};  // exterior states at this stage's time t + c_i dt
   return dispatch(g, [&](auto L) {
     using Lc = decltype(L);
-    timed(E, ES_KERNEL_PREP, st, [&] { Lc::prep(g.P, sp, g.aux, E.status, st, grid_for(E, g.N, 256)); });
+    timed(E, ES_KERNEL_PREP, st,
+          [&] { Lc::prep(g.P, sp, g.aux, E.status, st, grid_for(E, g.N, 256), g.any_bc ? &bc : nullptr); });
     timed(E, ES_KERNEL_FACE, st,
           [&] { Lc::face(g.P, g.aux, g.F, g.FL, st, grid_for(E, 3LL * g.K * g.P1 * g.P1, 256)); });
     if (ns) timed(E, ES_KERNEL_GRAD, st, [&] { Lc::grad(g.P, g.aux, g.fV, st, grid_for(E, g.N, 256)); });

@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "es_bc.cuh"
 #include "es_device.cuh"
 #include "es_face_fx.cuh"
 #include "es_launch.h"
@@ -410,11 +411,20 @@ __device__ __forceinline__ void stage_increment_w(const Params& P, const double 
 // FP64 selects the FP64-increment paths at compile time (they differ widely in
 // register use).  NPREV >= 0 fixes the number of earlier stages at compile time;
 // NPREV < 0 reads it from sp.nprev (tableaux with more than three nonzero a_ij in a row).
-template <typename TF, int NPREV, bool FP64>
-__global__ void k_prep(Params P, StagePrep sp, TF* __restrict__ aux, int* __restrict__ status) {
+// BC: the first block evaluates the exterior values of the boundaries instead (es_bc.cuh).
+template <typename TF, int NPREV, bool FP64, bool BC>
+__global__ void k_prep(Params P, StagePrep sp, TF* __restrict__ aux, int* __restrict__ status,
+                       const __grid_constant__ std::conditional_t<BC, BcEval, int> bc) {
+  if constexpr (BC) {
+    if (blockIdx.x == 0) {
+      for (int i = threadIdx.x >> 5; i < 6; i += blockDim.x >> 5) bc_eval_side(bc, i, threadIdx.x & 31);
+      return;
+    }
+  }
+  const int block = blockIdx.x - (BC ? 1 : 0), blocks = gridDim.x - (BC ? 1 : 0);
   const long long N = (long long)P.K * sp.Np;
   const double gam = P.gam;
-  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < N; g += (long long)gridDim.x * blockDim.x) {
+  for (long long g = block * (long long)blockDim.x + threadIdx.x; g < N; g += (long long)blocks * blockDim.x) {
     const int inst = inst_of(P, int(g / sp.Np));
     double u[5];
 #pragma unroll
@@ -1872,29 +1882,36 @@ inline int node_block(int& grid) {
   return 64;
 }
 
-template <typename TF, bool FP64>
-void prep_launch(const Params& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid) {
+template <typename TF, bool FP64, bool BC>
+void prep_launch(const Params& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid,
+                 const std::conditional_t<BC, BcEval, int>& bc) {
   const int nb = node_block(grid);
+  if (BC) ++grid;
   switch (sp.nprev) {
-    case 0: k_prep<TF, 0, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
-    case 1: k_prep<TF, 1, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
-    case 2: k_prep<TF, 2, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
-    case 3: k_prep<TF, 3, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
-    default: k_prep<TF, -1, FP64><<<grid, nb, 0, st>>>(P, sp, a, status); break;
+    case 0: k_prep<TF, 0, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
+    case 1: k_prep<TF, 1, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
+    case 2: k_prep<TF, 2, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
+    case 3: k_prep<TF, 3, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
+    default: k_prep<TF, -1, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
   }
+}
+template <typename TF, bool FP64>
+void prep_launch(const Params& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid, const BcEval* bc) {
+  if (bc) prep_launch<TF, FP64, true>(P, sp, a, status, st, grid, *bc);
+  else prep_launch<TF, FP64, false>(P, sp, a, status, st, grid, 0);
 }
 
 template <int P1, typename TF>
 void Launcher<P1, TF>::prep(const Params& P, const StagePrep& sp, void* aux, int* status, cudaStream_t st,
-                            int grid) {
+                            int grid, const BcEval* bc) {
   TF* a = static_cast<TF*>(aux);
   if constexpr (std::is_same<TF, double>::value) {
-    prep_launch<TF, true>(P, sp, a, status, st, grid);
+    prep_launch<TF, true>(P, sp, a, status, st, grid, bc);
   } else if constexpr (std::is_same<TF, float>::value) {
-    if (P.ff_est) prep_launch<TF, false>(P, sp, a, status, st, grid);
-    else prep_launch<TF, true>(P, sp, a, status, st, grid);
+    if (P.ff_est) prep_launch<TF, false>(P, sp, a, status, st, grid, bc);
+    else prep_launch<TF, true>(P, sp, a, status, st, grid, bc);
   } else {
-    prep_launch<TF, false>(P, sp, a, status, st, grid);
+    prep_launch<TF, false>(P, sp, a, status, st, grid, bc);
   }
 }
 

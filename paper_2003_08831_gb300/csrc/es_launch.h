@@ -97,9 +97,26 @@ constexpr int kGlobalRelaxIterations = 8;
 constexpr int kVolumeVariants = 3;
 constexpr int kStageVariants = 2 * kVolumeVariants;
 
+// Dirichlet-penalty boundary data of a context
+struct BcSpec {
+  int kind[3];           // ES_BC_* per direction
+  double q[3][2][5];     // ES_BC_STATE: exterior states (left, right)
+  double vs[3][6];       // ES_BC_VISCOUS_SHOCK: V_f, alpha, H, speed, x_lo, x_hi
+  double gam;
+};
+// the exterior values at time *t + t_off (0 + t_off without t) into out [3][2][kBcVals]
+struct BcEval {
+  BcSpec spec;
+  const double* t;
+  double t_off;
+  double* out;
+};
+
 template <int P1, typename TF>
 struct Launcher {
-  static void prep(const Params& P, const StagePrep& sp, void* aux, int* status, cudaStream_t st, int grid);
+  // bc: exterior values to be evaluated by the same launch (or null)
+  static void prep(const Params& P, const StagePrep& sp, void* aux, int* status, cudaStream_t st, int grid,
+                   const BcEval* bc = nullptr);
   // FL: -x_m boundary-face fluxes of the first elements along non-periodic directions (or null)
   static void face(const Params& P, const void* aux, void* F, void* FL, cudaStream_t st, int grid);
   static void grad(const Params& P, const void* aux, void* fV, cudaStream_t st, int grid);
