@@ -27,6 +27,7 @@ ES_HD bool fx_face_flux(const double a[5], const double b[5], int m, fx C1, int 
                         double f[5]) {
   const int h1a = fx_hi_word(a[0]), h1b = fx_hi_word(b[0]), h5a = fx_hi_word(a[4]), h5b = fx_hi_word(b[4]);
   int mxv = 0;
+#pragma unroll
   for (int k = 1; k < 4; ++k) {
     const int ha = fx_hi_word(a[k]) & 0x7fffffff, hb = fx_hi_word(b[k]) & 0x7fffffff;
     mxv = mxv > ha ? mxv : ha;
@@ -38,6 +39,7 @@ ES_HD bool fx_face_flux(const double a[5], const double b[5], int m, fx C1, int 
   // component order z1, z_m, the other two, z5
   fx x[2][5];
   FxPair p[2][2];
+#pragma unroll
   for (int s = 0; s < 2; ++s) {
     const double* z = s ? b : a;
     const double z0 = m == 0 ? z[1] : (m == 1 ? z[2] : z[3]), z1 = m == 0 ? z[2] : (m == 1 ? z[3] : z[1]),
@@ -60,6 +62,7 @@ ES_HD bool fx_face_flux(const double a[5], const double b[5], int m, fx C1, int 
     const fx c0 = sc.C - (1ll << (64 - sc.kt));  // 4/(gam-1) = C1x - 2
     const fx sg = fx(sqrt_gam * 0x1p60);
     fx lam = 0, rho[2], en[2];
+#pragma unroll
     for (int s = 0; s < 2; ++s) {
       const fx t = x[s][0] * 2;  // z1 as a fraction in [1/3, 1)
       const fx r = fx_rcp(t, fx_rcpf(float(unsigned(fx_hi(t))) * 0x1p-31f));           // 60 fractional bits
@@ -72,11 +75,13 @@ ES_HD bool fx_face_flux(const double a[5], const double b[5], int m, fx C1, int 
     }
     lam *= 4;                                                                          // 61
     D[0] = fx_product(lam, rho[1] - rho[0], E5 - 55);
+#pragma unroll
     for (int k = 1; k < 4; ++k)
       D[k] = fx_product(lam, fx_mul(x[1][4], x[1][k]) - fx_mul(x[0][4], x[0][k]), E5 - E1 + Ev - 55);
     D[4] = fx_product(lam, en[1] - en[0], E5 - 2 * E1 + sc.kt - 57);
   }
   double h[5];
+#pragma unroll
   for (int k = 0; k < 5; ++k) h[k] = fx_to_double(g[k], fx_unit(sc, k)) - D[k];
   f[0] = h[0];
   f[1] = m == 0 ? h[1] : (m == 1 ? h[3] : h[2]);

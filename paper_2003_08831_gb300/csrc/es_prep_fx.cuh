@@ -76,6 +76,7 @@ ES_HD bool fx_state(const double q[5], fx g1, int eg, FxState& z) {
   em = em > 673 ? em : 673;
   const fx nr = fx_from_positive(q[0], er), nE = fx_from_positive(q[4], eE);  // 2^61 .. 2^62
   fx nm[3];
+#pragma unroll
   for (int k = 0; k < 3; ++k) nm[k] = fx_from_double(q[1 + k], em);
   const int Er = er - 1022, EE = eE - 1022, Em = em - 1022;
   // rho E and |m|^2/2 in units of 2^(Er + EE - 60)
@@ -101,6 +102,7 @@ ES_HD bool fx_state(const double q[5], fx g1, int eg, FxState& z) {
   const int h = (ex - sh + 63) >> 1;
   const fx rs = fx_rsqrt(X);
   z.z1 = fx_mul(nr, rs);
+#pragma unroll
   for (int k = 0; k < 3; ++k) z.zv[k] = fx_mul(nm[k], rs);
   z.z5 = fx(fx_umulhi(uint64_t(X), uint64_t(rs)));
   z.s1 = Er + 1 - h;
@@ -118,6 +120,7 @@ ES_HD float fx_rcp_seed(fx f) {
 // the six planes of the parameter vector in FP64
 ES_HD void fx_state_planes(const FxState& z, double o[6]) {
   o[0] = fx_to_double(z.z1, z.s1 - 60);
+#pragma unroll
   for (int k = 0; k < 3; ++k) o[1 + k] = fx_to_double(z.zv[k], z.sv - 60);
   o[4] = fx_to_double(z.z5, z.s5 - 60);
   const fx f = z.z1 << 3;  // 2^61 .. 2^63
@@ -150,6 +153,7 @@ ES_HD bool fx_increment(const FxState& a, const FxState& b, fx C1, int ktg, doub
   const int ha = sv - a.sv < 63 ? sv - a.sv : 63, hb = sv - b.sv < 63 ? sv - b.sv : 63;
   const fx S1 = (a1 + b1) * 2, D1 = (b1 - a1) * 64;  // 61 and 66 fractional bits
   fx k2 = 0;
+#pragma unroll
   for (int k = 0; k < 3; ++k) {
     const fx av = a.zv[k] >> ha, bv = b.zv[k] >> hb;
     const fx S = av + bv, D = (bv - av) * 2;  // 60, 61
