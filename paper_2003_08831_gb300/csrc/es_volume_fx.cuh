@@ -14,8 +14,8 @@ namespace es {
 
 // High words of each element's extreme values: largest and smallest z1, z5, largest |z2..z4|.
 // kBad: a face flux or sum beyond the element's scales.
-// kRetry: the element is in its second attempt.
-enum { kMx1, kMn1, kMx5, kMn5, kMxV, kBad, kRetry, kFxMeta };
+// kRetry: the element is in its second attempt.  kMxT, kMxH: largest stress and viscous energy flux (NS).
+enum { kMx1, kMn1, kMx5, kMn5, kMxV, kBad, kRetry, kMxT, kMxH, kFxMeta };
 
 template <int P1, int EPB>
 struct VolFxSmem {
@@ -67,6 +67,16 @@ __device__ __forceinline__ bool warp_uniform(int v) {
 // largest biased exponent of the instance's metrics
 __device__ __forceinline__ int fx_metric_exponent(const InstGeom& G) {
   return max(max(__double2hiint(G.metric[0]), __double2hiint(G.metric[1])), __double2hiint(G.metric[2])) >> 20;
+}
+
+// Whether an element's viscous fluxes could leave its scales, from exponents: stress below mu |v| (2/h)/omega
+// 2^3, heat below kappa/R p/rho (2/h)/omega 2^1
+__device__ __forceinline__ bool fx_viscous_element(const Params& P, const FxScale& sc, int em) {
+  const int d = em - 1022 + P.fxKw, E1 = sc.e1 - 1022, v = sc.ev - 1022 - E1 + 1;
+  const int t = (__double2hiint(P.mu) >> 20) + d + v + 3;
+  const int h = (__double2hiint(P.kappa_heat * P.inv_R) >> 20) + 2 - 2 * E1 + d + 1;
+  const int room = sc.tier == kFxNear ? 1081 : 1080;
+  return t > room + fx_unit(sc, 1) || max(h, t + v) > room + fx_unit(sc, 4);
 }
 
 // An LGL line of an element outside the fixed-point range, in FP64 with its face terms (the
@@ -318,10 +328,42 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
       fx_smem_max(meta + kMxV * EPB + el, hv, one);
     }
     __syncthreads();
+    bool viscous = false;
     if (threadIdx.x < nel) {
       const int el = threadIdx.x;
       scale[el] = fx_scale(meta[kMx1 * EPB + el], meta[kMn1 * EPB + el], meta[kMx5 * EPB + el],
                            meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt, NS ? kFxViscous : kFxFine);
+      if constexpr (NS) viscous = fx_viscous_element(P, scale[el], fx_metric_exponent(geom_of(P, inst_of(P, e0 + el))));
+    }
+    // Where the viscous fluxes may not fit: looked at before any pair is formed, and the second
+    // attempt's scales at once if they do not (one that does not fit all the same is found below).
+    // Viscous shock 25^3 p = 3 693 -> 540 us per launch; looked at without the estimate before it, Navier--
+    // Stokes p = 4 takes 941 us (930 with, 924 with neither).
+    if constexpr (NS) {
+      if (__syncthreads_or(viscous)) {
+#pragma unroll 1
+        for (int t0 = 0; t0 < nn; t0 += THREADS) {
+          const int t = min(t0 + int(threadIdx.x), nn - 1), el = t / Np;
+          const double* f = fV + (long long)e0 * Np + t;
+          int top[2] = {0, 0};
+#pragma unroll
+          for (int c = 0; c < 12; ++c) {
+            int& h = top[(c & 3) == 3];
+            h = max(h, __double2hiint(f[c * N]) & 0x7fffffff);
+          }
+          const bool one = warp_uniform(el);
+          fx_smem_max(meta + kMxT * EPB + el, top[0], one);
+          fx_smem_max(meta + kMxH * EPB + el, top[1], one);
+        }
+        __syncthreads();
+        if (threadIdx.x < nel) {
+          const int el = threadIdx.x, room = scale[el].tier == kFxNear ? 1081 : 1080;  // volume_line_fx's limits
+          if ((meta[kMxT * EPB + el] >> 20) > room + fx_unit(scale[el], 1) ||
+              (meta[kMxH * EPB + el] >> 20) > room + fx_unit(scale[el], 4))
+            scale[el] = fx_scale(meta[kMx1 * EPB + el], meta[kMn1 * EPB + el], meta[kMx5 * EPB + el],
+                                 meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt, kFxCoarse);
+        }
+      }
     }
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
