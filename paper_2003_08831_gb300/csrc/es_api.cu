@@ -209,8 +209,8 @@ InstGeom instance_geom(const es_config& C, int off) {
 
 // Kernel parameters (LGL/SBP tables, metric, gas constants) of a configuration; host only,
 // no allocation.
-void build_params(const es_config& C, Params* out) {
-  Params& P = *out;
+void build_params(const es_config& C, FxParams* out) {
+  FxParams& P = *out;
   std::memset(&P, 0, sizeof(P));
   const int P1 = C.p + 1;
   double x[kMaxP1], w[kMaxP1], D[kMaxP1 * kMaxP1];
@@ -296,7 +296,7 @@ struct Group {
   long long N = 0;
   size_t tf = 8;  // bytes per flux value (8 FP64 and float-float, 4 mixed)
   bool ffx = false;  // float-float flux arithmetic (ES_FP64X)
-  Params P;
+  FxParams P;
   int vol_variant = 0;
   std::vector<InstGeom> geom;      // host copy of the instance table
   std::vector<int> inst_ids;       // batch instance index of each local instance
@@ -1046,7 +1046,7 @@ int es_relax_step(es_ctx* c, const double* u_old, const double* u_new, const dou
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Engine& E = c->eng;
   Group& g = c->g;
-  Params P = g.P;
+  FxParams P = g.P;
   P.g0.dt = 0.0;
   timed(E, ES_KERNEL_OTHER, st, [&] { launch_reset(g.gmin, g.pending, g.ninst, st); });
   StageRelax sr = relax_base(E, g);

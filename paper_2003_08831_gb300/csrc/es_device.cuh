@@ -65,12 +65,6 @@ struct Params {
   FluxConst<double> Cd;        // flux constants per precision (host-computed: no
   FluxConst<float> Cf;         // divisions or square roots in the kernels)
   FluxConst<ff> Cff;
-  // fixed-point tables of the FP64 volume term (es_fx.cuh)
-  long long fxQ[kMaxP1 * kMaxP1];  // omega_i D_ij / 4, 65 fractional bits
-  long long fxW[kMaxP1];           // 2^-fxKw / omega_i < 1, 63 fractional bits
-  long long fxC;                   // C1x 2^-fxKt < 1, 62 fractional bits
-  long long fxG;                   // gam - 1 = fxG 2^(fxEg - 63), 2^62 <= fxG < 2^63
-  int fxKt, fxKw, fxEg;
   int K;                       // elements in the group
   int diss;                    // Rusanov interface dissipation on/off
   int p1;                      // p + 1
@@ -84,6 +78,17 @@ struct Params {
   const double* bcz;           // device [3][2][kBcVals] exterior values (see kBcVals), or null
   const int* nbr;              // device [K][6]: periodic neighbour of each element along -x_m, +x_m
                                // (index 2 m + side), or null (then computed from the geometry)
+};
+
+// Params and the fixed-point tables (es_fx.cuh), for the kernels that use them: every launch copies
+// its arguments, and the float kernels of a step are short (mixed float-float Taylor--Green 32^3
+// p = 3: 3083 us for four steps with the first 364 of these bytes in Params, 3070 without).
+struct FxParams : Params {
+  long long fxQ[kMaxP1 * kMaxP1];  // omega_i D_ij / 4, 65 fractional bits
+  long long fxW[kMaxP1];           // 2^-fxKw / omega_i < 1, 63 fractional bits
+  long long fxC;                   // C1x 2^-fxKt < 1, 62 fractional bits
+  long long fxG;                   // gam - 1 = fxG 2^(fxEg - 63), 2^62 <= fxG < 2^63
+  int fxKt, fxKw, fxEg;
 };
 
 template <typename T> __device__ __forceinline__ const FluxConst<T>& flux_const(const Params& P);

@@ -83,7 +83,7 @@ enum { kGMx1, kGMn1, kGMxV, kGradMeta };
 
 template <int P1, int EPB, int THREADS>
 __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * 128))
-    k_grad_fx(const __grid_constant__ Params P, const double* __restrict__ aux, double* __restrict__ fV) {
+    k_grad_fx(const __grid_constant__ FxParams P, const double* __restrict__ aux, double* __restrict__ fV) {
   constexpr int P2 = P1 * P1, Np = P1 * P2, Nf = 6 * P2, ST = EPB * Np, SF = EPB * Nf;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx* ws = reinterpret_cast<fx*>(smem_raw);  // [4][ST] interior, [4][SF] outer states of the faces

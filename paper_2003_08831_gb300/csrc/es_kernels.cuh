@@ -395,7 +395,7 @@ static __device__ __noinline__ void increment_fp64(const double* u, const double
   entropy_var_increment(u, e, gam, inv_gm1, dw);
 }
 // w(y) - w(u), e = y - u up to y's rounding; zy: y's fixed-point state if it has one
-__device__ __forceinline__ void stage_increment_w(const Params& P, const double u[5], const double e[5],
+__device__ __forceinline__ void stage_increment_w(const FxParams& P, const double u[5], const double e[5],
                                                   const FxState* zy, double dw[5]) {
   FxState zu;
   if (zy && fx_state(u, P.fxG, P.fxEg, zu) && fx_increment(zu, *zy, P.fxC, P.fxKt, dw)) return;
@@ -413,7 +413,7 @@ __device__ __forceinline__ void stage_increment_w(const Params& P, const double 
 // NPREV < 0 reads it from sp.nprev (tableaux with more than three nonzero a_ij in a row).
 // BC: the first block evaluates the exterior values of the boundaries instead (es_bc.cuh).
 template <typename TF, int NPREV, bool FP64, bool BC>
-__global__ void k_prep(Params P, StagePrep sp, TF* __restrict__ aux, int* __restrict__ status,
+__global__ void k_prep(std::conditional_t<FP64, FxParams, Params> P, StagePrep sp, TF* __restrict__ aux, int* __restrict__ status,
                        const __grid_constant__ std::conditional_t<BC, BcEval, int> bc) {
   if constexpr (BC) {
     if (blockIdx.x == 0) {
@@ -652,10 +652,11 @@ static __device__ __noinline__ void face_flux_fp64(const Zstate<double>& L, doub
                                                    double* f) {
   face_flux(L, izL, R, izR, m, C, diss, f);
 }
+template <typename TF> using FaceParams = std::conditional_t<std::is_same<TF, double>::value, FxParams, Params>;
 // face_flux with k_face's constants: in FP64 mode through the fixed-point form (es_face_fx.cuh),
 // the matrix dissipation always in FP64
 template <typename TF>
-__device__ __forceinline__ void interface_flux(const Params& P, const FluxConst<TF>& C, const Zstate<TF>& L, TF izL,
+__device__ __forceinline__ void interface_flux(const FaceParams<TF>& P, const FluxConst<TF>& C, const Zstate<TF>& L, TF izL,
                                                const Zstate<TF>& R, TF izR, int m, TF f[5]) {
   if constexpr (std::is_same<TF, double>::value) {
     if (fx_face_flux(L.z, R.z, m, P.fxC, P.fxKt, C.sqrt_gam, P.diss, f)) {
@@ -671,7 +672,7 @@ __device__ __forceinline__ void interface_flux(const Params& P, const FluxConst<
 // VPEN: with the diss^V penalty (a separate instantiation keeps the common path's
 // register count)
 template <int P1, typename TF, bool VPEN>
-__device__ __forceinline__ void face_node(const Params& P, const FluxConst<TF>& C, const TF* __restrict__ aux,
+__device__ __forceinline__ void face_node(const FaceParams<TF>& P, const FluxConst<TF>& C, const TF* __restrict__ aux,
                                           TF* __restrict__ F, TF* __restrict__ FL, int e, int m, int ab) {
   constexpr int P2 = P1 * P1, Np = P1 * P2;
   const long long N = (long long)P.K * Np;
@@ -727,7 +728,7 @@ __global__ void k_face(Params P, const TF* __restrict__ aux, TF* __restrict__ F,
 // its dependent products.  Taylor--Green 32^3 p = 3 119 -> 102 us per launch, Navier--Stokes p = 4
 // 193 -> 162 us.  The other precisions keep the loop (float-float: 70 us; 84 in this form).
 template <int P1, bool VPEN>
-__global__ void __launch_bounds__(256, 3) k_face_fp64(const __grid_constant__ Params P, const double* __restrict__ aux,
+__global__ void __launch_bounds__(256, 3) k_face_fp64(const __grid_constant__ FxParams P, const double* __restrict__ aux,
                                                       double* __restrict__ F, double* __restrict__ FL) {
   constexpr unsigned P2 = P1 * P1;
   // (below 2^32 face nodes per direction: 2^32 are 700 GB of states)
@@ -1350,7 +1351,7 @@ __device__ __forceinline__ int group_max(int v, unsigned mask) {
 // Fixed-point solve of the element whose nodes the group holds; false: to the FP64 form.
 // T, Tf: the group's rows in shared memory.
 template <int P1>
-__device__ __forceinline__ bool relax_element_fx(const Params& P, const StageRelax& sr,
+__device__ __forceinline__ bool relax_element_fx(const FxParams& P, const StageRelax& sr,
                                                  const FxRelaxNode (&nd)[RelaxGroup<P1>::R], const double* w8, int sl,
                                                  unsigned gmask, double A, double J, fx* T, float* Tf, double& gk) {
   using RG = RelaxGroup<P1>;
@@ -1434,7 +1435,7 @@ __device__ __forceinline__ bool relax_element_fx(const Params& P, const StageRel
 
 // UNEW: the entry point that hands in u_new and d_eta
 template <int P1, bool UNEW>
-__global__ void __launch_bounds__(128, P1 == 6 ? 3 : 4) k_relax(const __grid_constant__ Params P, const __grid_constant__ StageRelax sr) {
+__global__ void __launch_bounds__(128, P1 == 6 ? 3 : 4) k_relax(const __grid_constant__ FxParams P, const __grid_constant__ StageRelax sr) {
   using RG = RelaxGroup<P1>;
   constexpr int Np = RG::Np, R = RG::R, SUB = RG::SUB;
   __shared__ double w8[Np];
@@ -1901,7 +1902,7 @@ inline int node_block(int& grid) {
 }
 
 template <typename TF, bool FP64, bool BC>
-void prep_launch(const Params& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid,
+void prep_launch(const FxParams& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid,
                  const std::conditional_t<BC, BcEval, int>& bc) {
   const int nb = node_block(grid);
   if (BC) ++grid;
@@ -1914,13 +1915,13 @@ void prep_launch(const Params& P, const StagePrep& sp, TF* a, int* status, cudaS
   }
 }
 template <typename TF, bool FP64>
-void prep_launch(const Params& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid, const BcEval* bc) {
+void prep_launch(const FxParams& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid, const BcEval* bc) {
   if (bc) prep_launch<TF, FP64, true>(P, sp, a, status, st, grid, *bc);
   else prep_launch<TF, FP64, false>(P, sp, a, status, st, grid, 0);
 }
 
 template <int P1, typename TF>
-void Launcher<P1, TF>::prep(const Params& P, const StagePrep& sp, void* aux, int* status, cudaStream_t st,
+void Launcher<P1, TF>::prep(const FxParams& P, const StagePrep& sp, void* aux, int* status, cudaStream_t st,
                             int grid, const BcEval* bc) {
   TF* a = static_cast<TF*>(aux);
   if constexpr (std::is_same<TF, double>::value) {
@@ -1934,7 +1935,7 @@ void Launcher<P1, TF>::prep(const Params& P, const StagePrep& sp, void* aux, int
 }
 
 template <int P1, typename TF>
-void Launcher<P1, TF>::face(const Params& P, const void* aux, void* F, void* FL, cudaStream_t st, int grid) {
+void Launcher<P1, TF>::face(const FxParams& P, const void* aux, void* F, void* FL, cudaStream_t st, int grid) {
   const int nb = node_block(grid);
   const TF* a = static_cast<const TF*>(aux);
   TF *f = static_cast<TF*>(F), *fl = static_cast<TF*>(FL);
@@ -1949,7 +1950,7 @@ void Launcher<P1, TF>::face(const Params& P, const void* aux, void* F, void* FL,
 }
 
 template <int P1, typename TF>
-void Launcher<P1, TF>::grad(const Params& P, const void* aux, void* fV, cudaStream_t st, int) {
+void Launcher<P1, TF>::grad(const FxParams& P, const void* aux, void* fV, cudaStream_t st, int) {
   if constexpr (std::is_same<TF, double>::value) {
     using C = GradFxCfg<P1>;
     const int grid = (P.K + C::EPB - 1) / C::EPB;
@@ -2002,7 +2003,7 @@ cudaError_t Launcher<P1, TF>::volume_setup() {
 }
 
 template <int P1, typename TF, int V>
-void volume_v(const Params& P, const StageVol& sv, const TF* aux, const TF* F, const TF* FL, const TF* fV, bool ns,
+void volume_v(const FxParams& P, const StageVol& sv, const TF* aux, const TF* F, const TF* FL, const TF* fV, bool ns,
               cudaStream_t st) {
   if constexpr (std::is_same<TF, double>::value) {
     using C = VolFxCfg<P1, V>;
@@ -2017,7 +2018,7 @@ void volume_v(const Params& P, const StageVol& sv, const TF* aux, const TF* F, c
 }
 
 template <int P1, typename TF>
-void Launcher<P1, TF>::volume(const Params& P, const StageVol& sv, const void* aux, const void* F, const void* FL, const void* fV,
+void Launcher<P1, TF>::volume(const FxParams& P, const StageVol& sv, const void* aux, const void* F, const void* FL, const void* fV,
                               bool ns, cudaStream_t st, int variant) {
   const TF* a = static_cast<const TF*>(aux);
   const TF* f = static_cast<const TF*>(F);
@@ -2069,7 +2070,7 @@ void Launcher<P1, TF>::volface(const Params& P, const StageVol& sv, const void* 
 }
 
 template <int P1, typename TF>
-void Launcher<P1, TF>::relax(const Params& P, const StageRelax& sr, cudaStream_t st, int grid) {
+void Launcher<P1, TF>::relax(const FxParams& P, const StageRelax& sr, cudaStream_t st, int grid) {
   // the u_new entry point (es_relax_step), the FP64 mode and the mixed mode with FP64
   // estimates solve in FP64; 4 warps per block, RelaxGroup::EPW elements per warp
   const bool fp64 = sr.u_new || std::is_same<TF, double>::value || (std::is_same<TF, float>::value && !P.ff_est);

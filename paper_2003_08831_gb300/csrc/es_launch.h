@@ -11,7 +11,7 @@ namespace es {
 // host helpers shared by the entry points (es_api.cu)
 int validate_config(const es_config& C);
 InstGeom instance_geom(const es_config& C, int off);
-void build_params(const es_config& C, Params* out);
+void build_params(const es_config& C, FxParams* out);
 int grid_for_sms(int sm_count, long long n, int block);
 void ff_split_host(double d, float out[2]);
 
@@ -115,19 +115,19 @@ struct BcEval {
 template <int P1, typename TF>
 struct Launcher {
   // bc: exterior values to be evaluated by the same launch (or null)
-  static void prep(const Params& P, const StagePrep& sp, void* aux, int* status, cudaStream_t st, int grid,
+  static void prep(const FxParams& P, const StagePrep& sp, void* aux, int* status, cudaStream_t st, int grid,
                    const BcEval* bc = nullptr);
   // FL: -x_m boundary-face fluxes of the first elements along non-periodic directions (or null)
-  static void face(const Params& P, const void* aux, void* F, void* FL, cudaStream_t st, int grid);
-  static void grad(const Params& P, const void* aux, void* fV, cudaStream_t st, int grid);
+  static void face(const FxParams& P, const void* aux, void* F, void* FL, cudaStream_t st, int grid);
+  static void grad(const FxParams& P, const void* aux, void* fV, cudaStream_t st, int grid);
   static cudaError_t volume_setup();
   // variant: volume tile (elements per CTA, threads), 0..kVolumeVariants-1
-  static void volume(const Params& P, const StageVol& sv, const void* aux, const void* F, const void* FL,
+  static void volume(const FxParams& P, const StageVol& sv, const void* aux, const void* F, const void* FL,
                      const void* fV, bool ns, cudaStream_t st, int variant);
   // k_volume with the interface fluxes evaluated in the kernel (TF = float, Euler, periodic)
   static cudaError_t volface_setup();
   static void volface(const Params& P, const StageVol& sv, const void* aux, cudaStream_t st, int variant);
-  static void relax(const Params& P, const StageRelax& sr, cudaStream_t st, int grid);
+  static void relax(const FxParams& P, const StageRelax& sr, cudaStream_t st, int grid);
   static void entropy(const Params& P, const double* q, double* eta, cudaStream_t st, int grid);
   // Theorem 2.3's eta_kappa(u) and estimate deta_kappa = sum P w(u).d - A (either output may be null)
   static void estimate(const Params& P, const double* q, const double* d, const double* A, double* eta_old,

@@ -107,7 +107,7 @@ extern "C" int es_rhs_noalloc(const es_config* cfg, const double* q, double* dqd
   int rc = setup_device(dev);
   if (rc != ES_OK) return rc;
 
-  Params P;
+  FxParams P;
   build_params(*cfg, &P);
   const bool fp64 = cfg->precision != ES_MIXED && cfg->precision != ES_MIXED_FF;
   const size_t tf = fp64 ? 8 : 4;

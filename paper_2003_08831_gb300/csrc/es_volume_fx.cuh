@@ -71,7 +71,7 @@ __device__ __forceinline__ int fx_metric_exponent(const InstGeom& G) {
 
 // Whether an element's viscous fluxes could leave its scales, from exponents: stress below mu |v| (2/h)/omega
 // 2^3, heat below kappa/R p/rho (2/h)/omega 2^1
-__device__ __forceinline__ bool fx_viscous_element(const Params& P, const FxScale& sc, int em) {
+__device__ __forceinline__ bool fx_viscous_element(const FxParams& P, const FxScale& sc, int em) {
   const int d = em - 1022 + P.fxKw, E1 = sc.e1 - 1022, v = sc.ev - 1022 - E1 + 1;
   const int t = (__double2hiint(P.mu) >> 20) + d + v + 3;
   const int h = (__double2hiint(P.kappa_heat * P.inv_R) >> 20) + 2 - 2 * E1 + d + 1;
@@ -147,7 +147,7 @@ __device__ __noinline__ void volume_line_fp64(const Params& P, const double* __r
 // (i = 0), the diagonal of D cancelling the lifting's interior half (fv: planes of this direction,
 // plane stride N; v_hi, v_lo: nodes whose values stand for f_next and f_prev).
 template <int P1, int TIER, bool NS, int DIRS>
-__device__ __forceinline__ bool volume_line_fx(const Params& P, const FxScale& sc, int m, int a, int b, fx wm,
+__device__ __forceinline__ bool volume_line_fx(const FxParams& P, const FxScale& sc, int m, int a, int b, fx wm,
                                                const fx* __restrict__ z, const float4* __restrict__ zf,
                                                const double* __restrict__ f_hi, const double* __restrict__ f_lo,
                                                long long fs, const double* __restrict__ fv, long long g0,
@@ -274,7 +274,7 @@ template <> struct VolFxCfg<6, kVolFxSmall> { static constexpr int EPB = 1, THRE
 
 // DIRS: directions worked on together, 1 (in turn, by the same threads) or 3 (small meshes)
 template <int P1, int EPB, int THREADS, int REGS, bool NS, int DIRS = 1>
-__global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx(const __grid_constant__ Params P,
+__global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx(const __grid_constant__ FxParams P,
                                                        const __grid_constant__ StageVol sv,
                                                        const double* __restrict__ aux, const double* __restrict__ F,
                                                        const double* __restrict__ FL,
