@@ -244,6 +244,7 @@ void build_params(const es_config& C, FxParams* out) {
   const long double gl = C.gamma_gas;
   P.fxG = llrintl(ldexpl(frexpl(gl - 1.0L, &P.fxEg), 63));
   if (P.fxG < 0) P.fxG = 0x7fffffffffffffffLL;  // rounded up to 2^63
+  P.fxI = llrintl(ldexpl(frexpl(1.0L / (gl - 1.0L), &P.fxEi), 62));
   P.fxC = llrintl(ldexpl(2.0L * (gl + 1.0L) / (gl - 1.0L), 62 - P.fxKt));
   P.kappa_heat = C.mu > 0.0 ? C.mu * C.gamma_gas * C.R / ((C.gamma_gas - 1.0) * C.Pr) : 0.0;
   P.K = C.nx * C.ny * C.nz;

@@ -88,7 +88,8 @@ struct FxParams : Params {
   long long fxW[kMaxP1];           // 2^-fxKw / omega_i < 1, 63 fractional bits
   long long fxC;                   // C1x 2^-fxKt < 1, 62 fractional bits
   long long fxG;                   // gam - 1 = fxG 2^(fxEg - 63), 2^62 <= fxG < 2^63
-  int fxKt, fxKw, fxEg;
+  long long fxI;                   // 1/(gam - 1) = fxI 2^(fxEi - 62), 2^61 <= fxI < 2^62
+  int fxKt, fxKw, fxEg, fxEi;
 };
 
 template <typename T> __device__ __forceinline__ const FluxConst<T>& flux_const(const Params& P);

@@ -28,6 +28,8 @@ typedef long long fx;
 
 #define ES_HD __host__ __device__ __forceinline__
 
+ES_HD int fx_max(int a, int b) { return a > b ? a : b; }
+ES_HD int fx_min(int a, int b) { return a < b ? a : b; }
 ES_HD int fx_lo(fx x) { return int(x); }
 ES_HD int fx_hi(fx x) { return int(x >> 32); }
 ES_HD fx fx_mulw(int a, int b) {

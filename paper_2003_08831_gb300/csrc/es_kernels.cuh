@@ -394,13 +394,6 @@ static __device__ __noinline__ void increment_fp64(const double* u, const double
                                                    double* dw) {
   entropy_var_increment(u, e, gam, inv_gm1, dw);
 }
-// w(y) - w(u), e = y - u up to y's rounding; zy: y's fixed-point state if it has one
-__device__ __forceinline__ void stage_increment_w(const FxParams& P, const double u[5], const double e[5],
-                                                  const FxState* zy, double dw[5]) {
-  FxState zu;
-  if (zy && fx_state(u, P.fxG, P.fxEg, zu) && fx_increment(zu, *zy, P.fxC, P.fxKt, dw)) return;
-  increment_fp64(u, e, P.gam, P.Cd.inv_gm1, dw);
-}
 
 // ---------------------------------------------------------------------------
 // y = u (+ gamma d when the instance has a pending relaxed update and this is the
@@ -412,16 +405,20 @@ __device__ __forceinline__ void stage_increment_w(const FxParams& P, const doubl
 // register use).  NPREV >= 0 fixes the number of earlier stages at compile time;
 // NPREV < 0 reads it from sp.nprev (tableaux with more than three nonzero a_ij in a row).
 // BC: the first block evaluates the exterior values of the boundaries instead (es_bc.cuh).
+template <bool FP64> using PrepParams = std::conditional_t<FP64, FxParams, Params>;
+template <bool BC> using PrepBc = std::conditional_t<BC, BcEval, int>;
 template <typename TF, int NPREV, bool FP64, bool BC>
-__global__ void k_prep(std::conditional_t<FP64, FxParams, Params> P, StagePrep sp, TF* __restrict__ aux, int* __restrict__ status,
-                       const __grid_constant__ std::conditional_t<BC, BcEval, int> bc) {
+__device__ __forceinline__ void prep_body(const PrepParams<FP64>& P, const StagePrep& sp, TF* __restrict__ aux,
+                                          int* __restrict__ status, const PrepBc<BC>& bc) {
   if constexpr (BC) {
     if (blockIdx.x == 0) {
-      for (int i = threadIdx.x >> 5; i < 6; i += blockDim.x >> 5) bc_eval_side(bc, i, threadIdx.x & 31);
+      for (int i = threadIdx.x >> 5; i < 6 && blockIdx.y == 0; i += blockDim.x >> 5) bc_eval_side(bc, i, threadIdx.x & 31);
       return;
     }
   }
   const int block = blockIdx.x - (BC ? 1 : 0), blocks = gridDim.x - (BC ? 1 : 0);
+  // with two rows of blocks the second forms the increments, the first all else
+  const bool planes = blockIdx.y == 0, increments = sp.dw && (gridDim.y == 1 || blockIdx.y == 1);
   const long long N = (long long)P.K * sp.Np;
   const double gam = P.gam;
   for (long long g = block * (long long)blockDim.x + threadIdx.x; g < N; g += (long long)blocks * blockDim.x) {
@@ -440,17 +437,16 @@ __global__ void k_prep(std::conditional_t<FP64, FxParams, Params> P, StagePrep s
     if constexpr (FP64 && !std::is_same<TF, double>::value) {
       double e[5];
       stage_increment_f64<TF, NPREV>(P, sp, N, g, inst, e);
-      TF z[6];
-      if (!stage_z_f64<TF>(P, u, e, z)) atomicOr(status, kStatusNonphysical);
+      if (planes) {
+        TF z[6];
+        if (!stage_z_f64<TF>(P, u, e, z)) atomicOr(status, kStatusNonphysical);
 #pragma unroll
-      for (int c = 0; c < 6; ++c) aux[c * N + g] = z[c];
-      if (sp.dw) {
-        double y[5], dw[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) y[v] = u[v] + e[v];
-        FxState zy;
-        const bool ok = fx_state(y, P.fxG, P.fxEg, zy);
-        stage_increment_w(P, u, e, ok ? &zy : nullptr, dw);
+        for (int c = 0; c < 6; ++c) aux[c * N + g] = z[c];
+      }
+      if (increments) {
+        double dw[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // (no earlier stage: y = u)
+        if constexpr (NPREV != 0)
+          if (!fx_increment(u, e, P.fxC, P.fxKt, P.fxI, P.fxEi, dw)) increment_fp64(u, e, P.gam, P.Cd.inv_gm1, dw);
 #pragma unroll
         for (int v = 0; v < 5; ++v) sp.dw[v * N + g] = dw[v];
       }
@@ -468,20 +464,36 @@ __global__ void k_prep(std::conditional_t<FP64, FxParams, Params> P, StagePrep s
           for (int v = 0; v < 5; ++v) y[v] = fma(c, kj[v * N + g], y[v]);
         }
       }
-      double z[6];
-      FxState zy;
-      const bool ok = fx_state(y, P.fxG, P.fxEg, zy);
-      if (ok) fx_state_planes(zy, z);
-      else if (!param_vector_fp64(y, gam, z)) atomicOr(status, kStatusNonphysical);
+      FxBase b;
+      const bool ok = fx_base(y, b);
+      if (increments) {  // (from y back to u, the fractions of y being at hand)
+        double e[5], dw[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-      for (int c = 0; c < 6; ++c) aux[c * N + g] = z[c];
-      if (sp.dw) {
-        double e[5], dw[5];
+        for (int v = 0; v < 5; ++v) e[v] = u[v] - y[v];
+        if constexpr (NPREV != 0) {
+          if (ok && fx_increment(b, e, P.fxC, P.fxKt, P.fxI, P.fxEi, dw)) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) e[v] = y[v] - u[v];
-        stage_increment_w(P, u, e, ok ? &zy : nullptr, dw);
+            for (int v = 0; v < 5; ++v) dw[v] = -dw[v];
+          } else {
+#pragma unroll
+            for (int v = 0; v < 5; ++v) e[v] = -e[v];
+            increment_fp64(u, e, P.gam, P.Cd.inv_gm1, dw);
+          }
+        }
 #pragma unroll
         for (int v = 0; v < 5; ++v) sp.dw[v * N + g] = dw[v];
+      }
+      if (planes) {
+        double z[6];
+        FxState zy;
+        if (ok) {
+          fx_parameters(b, P.fxG, P.fxEg, zy);
+          fx_state_planes(zy, z);
+        } else if (!param_vector_fp64(y, gam, z)) {
+          atomicOr(status, kStatusNonphysical);
+        }
+#pragma unroll
+        for (int c = 0; c < 6; ++c) aux[c * N + g] = z[c];
       }
     } else {
       ff uf[5], ef[5];
@@ -498,6 +510,19 @@ __global__ void k_prep(std::conditional_t<FP64, FxParams, Params> P, StagePrep s
       }
     }
   }
+}
+template <typename TF, int NPREV, bool FP64, bool BC>
+__global__ void k_prep(PrepParams<FP64> P, StagePrep sp, TF* __restrict__ aux, int* __restrict__ status,
+                       const __grid_constant__ PrepBc<BC> bc) {
+  prep_body<TF, NPREV, FP64, BC>(P, sp, aux, status, bc);
+}
+// with the fixed-point increment: four blocks of 256 threads per SM.  Taylor--Green 32^3 p = 3, later
+// and first stages: 154 and 70 us (three or five blocks: 2 and 20 % longer); ES_MIXED p = 4 24^3, later stages: 135
+// (three blocks 144).
+template <typename TF, int NPREV, bool FP64, bool BC>
+__global__ void __launch_bounds__(256, 4) k_prep_capped(PrepParams<FP64> P, StagePrep sp, TF* __restrict__ aux,
+                                                        int* __restrict__ status, const __grid_constant__ PrepBc<BC> bc) {
+  prep_body<TF, NPREV, FP64, BC>(P, sp, aux, status, bc);
 }
 
 // ---------------------------------------------------------------------------
@@ -1906,12 +1931,20 @@ void prep_launch(const FxParams& P, const StagePrep& sp, TF* a, int* status, cud
                  const std::conditional_t<BC, BcEval, int>& bc) {
   const int nb = node_block(grid);
   if (BC) ++grid;
+  // Small meshes wait for the chain of a node's operations: parameter vector and increment by different
+  // threads (isentropic vortex 4^3 p = 3: 5.2 -> 4.8 us per launch).
+  const dim3 blocks(grid, FP64 && nb == 64 && sp.dw && !sp.pending ? 2 : 1);
+  const auto launch = [&](auto n) {
+    constexpr int NPREV = decltype(n)::value;
+    if constexpr (FP64 && (NPREV != 0 || std::is_same<TF, double>::value)) k_prep_capped<TF, NPREV, FP64, BC><<<blocks, nb, 0, st>>>(P, sp, a, status, bc);
+    else k_prep<TF, NPREV, FP64, BC><<<blocks, nb, 0, st>>>(P, sp, a, status, bc);
+  };
   switch (sp.nprev) {
-    case 0: k_prep<TF, 0, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
-    case 1: k_prep<TF, 1, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
-    case 2: k_prep<TF, 2, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
-    case 3: k_prep<TF, 3, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
-    default: k_prep<TF, -1, FP64, BC><<<grid, nb, 0, st>>>(P, sp, a, status, bc); break;
+    case 0: launch(std::integral_constant<int, 0>{}); break;
+    case 1: launch(std::integral_constant<int, 1>{}); break;
+    case 2: launch(std::integral_constant<int, 2>{}); break;
+    case 3: launch(std::integral_constant<int, 3>{}); break;
+    default: launch(std::integral_constant<int, -1>{}); break;
   }
 }
 template <typename TF, bool FP64>

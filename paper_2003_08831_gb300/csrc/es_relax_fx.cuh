@@ -42,8 +42,6 @@ ES_HD fx fx_inv_table(int k) {
 #endif
 }
 
-ES_HD int fx_max(int a, int b) { return a > b ? a : b; }
-ES_HD int fx_min(int a, int b) { return a < b ? a : b; }
 ES_HD fx fx_abs(fx x) { return x < 0 ? -x : x; }
 // x 2^s; to the left only where the result fits
 ES_HD fx fx_shift(fx x, int s) {
