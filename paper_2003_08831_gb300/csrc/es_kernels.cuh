@@ -1391,7 +1391,10 @@ __device__ __forceinline__ bool relax_element_fx(const FxParams& P, const StageR
   bits = group_max<SUB>(bits, gmask);
   er = group_max<SUB>(er, gmask);
   const int E = bits + 2;
-  if (E < kRelaxMinE || E > kRelaxMaxE) return false;
+  gk = __longlong_as_double(0x7ff0000000000000LL);  // +inf: unconstrained
+  // (elements that hardly change: a free stream, gas at rest)
+  if (E < kRelaxMinE) return fx_relax_below_floor(bits, sr.delta_floor, P.Cd.inv_gm1);
+  if (E > kRelaxMaxE) return false;
   FxRelaxTerm t[R];
   fx cd[R];
   int ex[R];
@@ -1410,13 +1413,14 @@ __device__ __forceinline__ bool relax_element_fx(const FxParams& P, const StageR
   const float lhs = 2.0f * est * fx_pow2(2 * E);
   const float rhs = float(sr.delta_floor * sr.delta_floor * P.Cd.gm1) * cs;
   if (!(est > 1e-30f)) return false;
-  gk = __longlong_as_double(0x7ff0000000000000LL);  // +inf: unconstrained
   if (lhs < 0.999f * rhs) return true;               // (an infinite floor too: relaxation switched off)
   if (!(lhs > 1.001f * rhs)) return false;
   if (!(A < 0.0)) {
     if (sl == 0) atomicOr(sr.status, kStatusNoRoot);
     return true;
   }
+  // (a root that fx_relax_root will not take: the series are not worth forming)
+  if (!fx_relax_near_one(est, E, er, A, J, P.fxG, P.fxEg)) return false;
   const int unit = fx_relax_unit(est), kl = fx_relax_last(E), kf = fx_relax_first_f(E);
   const fx gp1 = fx_relax_gp1(P.fxG, P.fxEg);
   FxRelaxSeries s[R];

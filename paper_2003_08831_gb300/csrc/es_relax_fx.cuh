@@ -139,6 +139,14 @@ ES_HD int fx_relax_bits(const FxRelaxNode& n) {
   return fx_max(fx_max(bx, by), bw);
 }
 
+// Whether |X|, |Y|, sqrt(W) < 2^bits alone keep the element's RMS change
+//   2 a/sum c <= max (X^2 + ((X - Y)^2 + 2 W)/(gam-1)) < 2^(2 bits) (1 + 6/(gam-1))
+// below the floor (a 1/1000 of room for the rounding of the FP64 form's sums; increments below 2^-499 read as 0)
+ES_HD bool fx_relax_below_floor(int bits, double floor, double inv_gm1) {
+  const double top = fx_make_double(uint64_t(1023 + 2 * fx_max(bits, -490)) << 52) * (1.001 + 6.006 * inv_gm1);
+  return floor * floor >= top;
+}
+
 // The node's mass weight c = cn 2^ce, cn in 2^60 .. 2^62 (w8 = omega_i omega_j omega_k/8, er: the
 // element's largest density exponent; c sums to less than 1/2), and X, Y as fractions of 2^E (E =
 // s + 2: below 1/4), W of 2^2E, with 64 fractional bits.
@@ -165,6 +173,15 @@ ES_HD fx fx_relax_d2(const FxRelaxNode& n, const FxRelaxTerm& t, int s, int E, f
                fx_shift(n.w, n.ew - 2 * En + 64);
   *ex = t.ce - 1 + 2 * (En - E);
   return fx_mul63(t.cn, D);
+}
+ES_HD float fx_int_float(int i) {
+#ifdef __CUDA_ARCH__
+  return __int_as_float(i);
+#else
+  float f;
+  __builtin_memcpy(&f, &i, 4);
+  return f;
+#endif
 }
 // 2^n as a float, 0 below the normal range (n <= 127)
 ES_HD float fx_pow2(int n) {
@@ -214,6 +231,16 @@ ES_HD fx fx_relax_gp1(fx g1, int eg) { return (g1 >> (2 - eg)) + (1ll << 62); }
 ES_HD fx fx_relax_coefficient(int k, fx sp, fx sm, fx sx, fx gp1) {
   const fx ik = fx_inv_table(k), i1 = fx_inv_table(k - 1);
   return fx_mul63(fx_mul(sp << 3, gp1), i1 - ik) - fx_mul63(sm, ik) + fx_mul63(sx, i1);
+}
+// Whether fx_relax_root's q, from the sum's FP32 estimate, can lie in its range 0.5 .. 1.5
+ES_HD bool fx_relax_near_one(float est, int E, int er, double A, double J, fx g1, int eg) {
+  const auto mantissa = [](int h) { return fx_int_float((h & 0xfffff) << 3 | 0x3f800000); };
+  const int hA = fx_hi_word(A) & 0x7fffffff, hJ = fx_hi_word(J), he = fx_bits(est);
+  const float f = fx_mulf(fx_mulf(mantissa(hA), fx_fraction(g1) * 4.0f), fx_rcpf(fx_mulf(mantissa(hJ), fx_int_float((he & 0x7fffff) | 0x3f800000))));
+  const int n = (hA >> 20) - (hJ >> 20) - ((he >> 23) - 127) + eg - 1 - 2 * E - er - 4;  // q = f 2^n
+  if (n < -4 || n > 4) return false;
+  const float q = fx_mulf(f, fx_pow2(n));
+  return q > 0.499f && q < 1.501f;
 }
 struct FxRelaxSeriesF {
   float x, al, be, p, m, mb;
