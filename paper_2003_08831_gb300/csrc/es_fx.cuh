@@ -288,9 +288,12 @@ struct FxScale {
 // 20 fraction bits are all ones, so that the sum of two fractions stays below 1 - 2^-20 (the upper
 // limb of fx_mul rounds up)
 ES_HD int fx_block_exponent(int mx) { return (mx + 1) >> 20; }
+// (of the velocities down to the slowest block that is taken, |z_v| = 2^-30: a block exponent that
+// stopped above it would cost the mass and energy flux, which are proportional to the velocity, their digits)
+constexpr int kFxSlowest = 993;
 ES_HD int fx_block_exponent_v(int mxv) {
   const int e = fx_block_exponent(mxv);
-  return e > 1007 ? e : 1007;
+  return e > kFxSlowest ? e : kFxSlowest;
 }
 
 // Room in the momentum and energy sums beyond the element's own fluxes: none; kFxViscous: the energy
@@ -312,7 +315,7 @@ ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int k
   s.e5 = fx_block_exponent(mx5);
   s.ev = fx_block_exponent_v(mxv);
   const bool ok = mn1 > 0 && mn5 > 0 && s.e1 > 822 && s.e1 < 1222 && s.e5 > 822 && s.e5 < 1222 && s.ev <= 1024 &&
-                  (mxv >> 20) >= 993 && ktg <= 12 && (mx1 >> 20) - (mn1 >> 20) <= 1 && (mx5 >> 20) - (mn5 >> 20) <= 1;
+                  (mxv >> 20) >= kFxSlowest && ktg <= 12 && (mx1 >> 20) - (mn1 >> 20) <= 1 && (mx5 >> 20) - (mn5 >> 20) <= 1;
   // 21 leading bits of largest and smallest: (max - min)/(max + min) <= 0.2 or 0.01
   const int a1 = (mx1 & 0xfffff) | 0x100000, b1 = ((mn1 & 0xfffff) | 0x100000) >> (((mx1 >> 20) - (mn1 >> 20)) & 1);
   const int a5 = (mx5 & 0xfffff) | 0x100000, b5 = ((mn5 & 0xfffff) | 0x100000) >> (((mx5 >> 20) - (mn5 >> 20)) & 1);
@@ -325,7 +328,7 @@ ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int k
   s.sp = (Ev > 0 ? 2 * Ev : 0) + c;
   s.se = room == kFxFine ? 0 : (room == kFxCoarse ? (Ev < 0 ? -Ev : 0) + 6 : (Ev < -4 ? -Ev - 4 : 0));
   s.kt = (ktg > 2 * Ev + 3 ? ktg : 2 * Ev + 3) + 1;
-  s.ss = s.kt - 2 - 2 * Ev;
+  s.ss = fx_min(s.kt - 2 - 2 * Ev, 63);
   s.C = (C1 >> ((s.kt - 1 - ktg) & 63));
   return s;
 }

@@ -1,0 +1,105 @@
+// Host check of the fixed-point two-point flux (csrc/es_fx.cuh) at the edges of its range.
+//   slow  gas slower than the velocities' other scales: mass and energy flux relative to themselves
+#include <algorithm>
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <random>
+
+#include "es_fx.cuh"
+
+using namespace es;
+typedef long double L;
+
+static L series(L r) {
+  L s = 0;
+  for (int k = 14; k >= 0; --k) s = s * r * r + 1.0L / (2 * k + 1);
+  return s;
+}
+static void flux(const double* p, const double* q, L gam, L f[5]) {  // z1, z_m, z_a, z_b, z5
+  L a[5], b[5];
+  for (int k = 0; k < 5; ++k) a[k] = p[k], b[k] = q[k];
+  const L s1 = a[0] + b[0], s5 = a[4] + b[4];
+  const L f1 = series((a[0] - b[0]) / s1), g = 1 / series((a[4] - b[4]) / s5);
+  const L u = (a[1] + b[1]) / s1, v = (a[2] + b[2]) / s1, w = (a[3] + b[3]) / s1, p1 = s5 / s1;
+  const L m = s1 * s5 * g / 4 * u;
+  f[0] = m;
+  f[1] = m * u + p1;
+  f[2] = m * v;
+  f[3] = m * w;
+  f[4] = u * gam / (gam - 1) * p1 * ((gam + 1) / (2 * gam) * g * f1 + (gam - 1) / (2 * gam)) + m * (u * u + v * v + w * w) / 2;
+}
+
+struct Gas {
+  fx C1;
+  int kt = 0;
+  explicit Gas(double gam) {
+    const L c = 2 * ((L)gam + 1) / ((L)gam - 1);
+    while (ldexpl(1, kt) <= c) ++kt;
+    C1 = llrintl(ldexpl(c, 62 - kt));
+  }
+};
+
+// |difference| of the pair's flux from long double beyond the result's rounding, Q |Q_ij|/4 with 65 bits;
+// false outside the range
+static bool pair(const double a[5], const double b[5], double gam, const Gas& gas, fx Q, L diff[5], L want[5], FxScale& s) {
+  int mxv = 0;
+  for (int k = 1; k < 4; ++k)
+    mxv = std::max({mxv, fx_hi_word(a[k]) & 0x7fffffff, fx_hi_word(b[k]) & 0x7fffffff});
+  s = fx_scale(std::max(fx_hi_word(a[0]), fx_hi_word(b[0])), std::min(fx_hi_word(a[0]), fx_hi_word(b[0])),
+               std::max(fx_hi_word(a[4]), fx_hi_word(b[4])), std::min(fx_hi_word(a[4]), fx_hi_word(b[4])), mxv, gas.C1, gas.kt);
+  if (s.tier == kFxSlow) return false;
+  fx x[2][5], g[5];
+  FxPair p[2][2];
+  for (int i = 0; i < 2; ++i) {
+    const double* z = i ? b : a;
+    x[i][0] = fx_from_positive(z[0], s.e1);
+    x[i][4] = fx_from_positive(z[4], s.e5);
+    for (int k = 1; k < 4; ++k) x[i][k] = fx_from_double(z[k], s.ev);
+    p[i][0] = fx_pair(x[i][0]);
+    p[i][1] = fx_pair(x[i][4]);
+  }
+  if (s.tier == kFxNear) fx_flux<kFxNear>(x[0], p[0], x[1], p[1], Q, s, g);
+  else fx_flux<kFxFar>(x[0], p[0], x[1], p[1], Q, s, g);
+  flux(a, b, gam, want);
+  for (int v = 0; v < 5; ++v) {
+    want[v] *= ldexpl((L)Q, -65) * 8;
+    diff[v] = fabsl(ldexpl((L)g[v], fx_unit(s, v)) - want[v]) - ldexpl(fabsl(want[v]), -53);
+  }
+  return true;
+}
+
+int main(int argc, char** argv) {
+  std::mt19937_64 R(31);
+  std::uniform_real_distribution<double> U(-1, 1);
+  L diff[5], want[5];
+  FxScale s;
+  if (!strcmp(argv[1], "slow"))
+    for (double gam : {1.4, 5.0 / 3.0, 1.1, 4.0})
+      for (double speed : {1e-3, 1e-5, 1e-6, 1e-7, 1e-8, 2e-9})
+        for (double var : {0.0, 1e-4, 0.1}) {
+          const Gas gas(gam);
+          L mass = 0, energy = 0;
+          int out = 0;
+          for (int it = 0; it < 4000; ++it) {
+            double z[2][5];
+            const double z1 = exp(6 * U(R)), z5 = exp(6 * U(R)), v = speed * (1 + fabs(U(R)));
+            for (auto& n : z) {
+              n[0] = z1 * (1 - var * fabs(U(R)));
+              n[4] = z5 * (1 - var * fabs(U(R)));
+              n[1] = v * (1 + var * U(R));  // along the line
+              n[2] = v * U(R);
+              n[3] = v * U(R);
+            }
+            const fx Q = fx(ldexp(0.25 * (0.25 + 0.7 * fabs(U(R))), 62)) * 8 * (it % 2 ? 1 : -1);
+            if (!pair(z[0], z[1], gam, gas, Q, diff, want, s)) {
+              ++out;
+              continue;
+            }
+            mass = std::max(mass, diff[0] / fabsl(want[0]));
+            energy = std::max(energy, diff[4] / fabsl(want[4]));
+          }
+          printf("slow %g %g %g out %d mass %.2Lf energy %.2Lf\n", gam, speed, var, out, ldexpl(mass, 53), ldexpl(energy, 53));
+        }
+  return 0;
+}

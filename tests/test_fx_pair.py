@@ -1,0 +1,38 @@
+"""The fixed-point two-point flux (csrc/es_fx.cuh) at the edges of its range, on the host against long double.
+
+Bounds.
+* Slow gas: the factors of mass and energy flux carry units of 2^-62 of the block scale, 64 of them in all
+  (tests/test_fx_flux.py); with |Q_ij| >= 1/4, velocity and z5 at least half of their blocks' the mass flux is above
+  2^-4 of the scale and the energy flux above 2^-6, so 64 units are 2 and 8 units of 2^-53 of the flux itself.
+"""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+
+
+@pytest.fixture(scope="module")
+def check(tmp_path_factory):
+    if not os.path.exists(NVCC):
+        pytest.skip("nvcc not found")
+    exe = str(tmp_path_factory.mktemp("fx") / "check")
+    subprocess.run([NVCC, "-std=c++17", "--expt-relaxed-constexpr", "-w", "-O2", "-I",
+                    os.path.join(ROOT, "paper_2003_08831_gb300", "csrc"), "-o", exe,
+                    os.path.join(ROOT, "tests", "fx_pair_check.cu")], check=True)
+
+    def run(part):
+        out = subprocess.run([exe, part], check=True, capture_output=True, text=True).stdout
+        return [ln.split() for ln in out.splitlines()]
+    return run
+
+
+def test_slow_gas(check):
+    rows = check("slow")
+    assert len(rows) == 4 * 6 * 3
+    for ln in rows:
+        assert int(ln[5]) == 0, ln
+        assert float(ln[7]) <= 2.0 and float(ln[9]) <= 8.0, ln
