@@ -296,20 +296,13 @@ ES_HD int fx_block_exponent_v(int mxv) {
   return e > kFxSlowest ? e : kFxSlowest;
 }
 
-// Room in the momentum and energy sums beyond the element's own fluxes: none; kFxViscous: the energy
-// sum's unit follows the velocity scale only down to Mach ~1/16 (heat conduction does not vanish
-// with the velocity); kFxCoarse: face and viscous fluxes up to 2^6 times the pressure and the
-// enthalpy flux at sound speed (the second attempt of an element that did not fit).
-constexpr int kFxFine = 0, kFxViscous = 1, kFxCoarse = 2;
-
 // From the high words of the element's largest and smallest z1 and z5 and largest |z2..z4|.
 // Fast when z1 and z5 are positive and vary by less than a factor 1.5 (u <= 0.04 for every
 // pair; NaN, infinities and signs fall through the comparisons of the high words), their
 // exponents leave every product inside the double range, and |z_v| < 4 (Mach below ~3.4).  Gas at
 // rest (|z_v| < 2^-30) stays in FP64: there the volume sums have to cancel the face fluxes' bits
 // (what remains is all that an undisturbed element next to a discontinuity moves by).
-ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int ktg,
-                       int room = kFxFine) {
+ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int ktg) {
   FxScale s;
   s.e1 = fx_block_exponent(mx1);
   s.e5 = fx_block_exponent(mx5);
@@ -323,14 +316,27 @@ ES_HD FxScale fx_scale(int mx1, int mn1, int mx5, int mn5, int mxv, fx C1, int k
   const bool near = (a1 - b1 + 1) * 100 <= a1 + b1 && (a5 - b5 + 1) * 100 <= a5 + b5;
   s.tier = !(ok && far) ? kFxSlow : (near ? kFxNear : kFxFar);
   const int Ev = s.ev - 1022;
-  const int c = room == kFxCoarse ? 6 : 0;
-  s.sv = (Ev < 0 ? -2 * Ev : 0) + c;
-  s.sp = (Ev > 0 ? 2 * Ev : 0) + c;
-  s.se = room == kFxFine ? 0 : (room == kFxCoarse ? (Ev < 0 ? -Ev : 0) + 6 : (Ev < -4 ? -Ev - 4 : 0));
+  s.sv = Ev < 0 ? -2 * Ev : 0;
+  s.sp = Ev > 0 ? 2 * Ev : 0;
+  s.se = 0;
   s.kt = (ktg > 2 * Ev + 3 ? ktg : 2 * Ev + 3) + 1;
   s.ss = fx_min(s.kt - 2 - 2 * Ev, 63);
   s.C = (C1 >> ((s.kt - 1 - ktg) & 63));
   return s;
+}
+// More room in the momentum and the energy sums, for an element whose face or viscous fluxes pass its
+// scales by 2^dm and 2^de.  The room is taken from the last bits of all its sums: as much as those fluxes need, and
+// kFxMargin bits beside it (of the five that the sums have over a double's), so that larger ones found later
+// do not take another attempt.  Up to 2^6 times the pressure and the enthalpy flux at sound speed, else FP64.
+constexpr int kFxMargin = 3;
+ES_HD void fx_widen(FxScale& s, int dm, int de) {
+  const int Ev = s.ev - 1022;
+  if (dm > 0) dm = fx_max(dm, fx_min(dm + kFxMargin, (Ev > 0 ? 2 * Ev : 0) + 6 - s.sp));
+  if (de > 0) de = fx_max(de, fx_min(de + kFxMargin, (Ev < 0 ? -Ev : 0) + 6 - s.se));
+  s.sv = fx_min(s.sv + dm, 63);
+  s.sp += dm;
+  s.se += de;
+  if (s.sp > (Ev > 0 ? 2 * Ev : 0) + 6 || s.se > (Ev < 0 ? -Ev : 0) + 6) s.tier = kFxSlow;
 }
 // exponents of the flux sums' units: 2 Q_ij times the flux is n 2^unit for mass, momentum and energy
 ES_HD int fx_unit(const FxScale& s, int v) {

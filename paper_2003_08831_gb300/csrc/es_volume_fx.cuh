@@ -13,9 +13,11 @@
 namespace es {
 
 // High words of each element's extreme values: largest and smallest z1, z5, largest |z2..z4|.
-// kBad: a face flux or sum beyond the element's scales.
-// kRetry: the element is in its second attempt.  kMxT, kMxH: largest stress and viscous energy flux (NS).
+// kBad: a face flux, viscous flux or sum beyond the element's scales (kFxMass: a mass flux).
+// kRetry: the element is in its second attempt.  kMxT, kMxH: bits by which its momentum and energy fluxes pass
+// the scales (before the lines, for Navier--Stokes: largest stress and viscous energy flux).
 enum { kMx1, kMn1, kMx5, kMn5, kMxV, kBad, kRetry, kMxT, kMxH, kFxMeta };
+constexpr int kFxWide = 1, kFxMass = 2;
 
 template <int P1, int EPB>
 struct VolFxSmem {
@@ -139,20 +141,21 @@ __device__ __noinline__ void volume_line_fp64(const Params& P, const double* __r
 // One LGL line in fixed point: every unordered pair once, both nodes' sums in registers, the
 // face fluxes at both ends (f_hi, f_lo: plane stride fs), for Navier--Stokes the viscous
 // divergence, then each node's sum times metric/omega_i into the element's accumulator.  Component order (z1, z_m, the other two, z5),
-// so that the flux needs no selects on the direction.  Returns false when a face flux (2^60, near:
-// 2^61), a viscous flux (2^58, 2^59) or a sum (2^61: the weighted sums of three directions stay
-// below 2^63) does not fit the element's scales; with the bounds of fx_flux no sum passes 2^63
-// before it is checked.
+// so that the flux needs no selects on the direction.  Returns 0, or what does not
+// fit the element's scales (kFxMass, kFxWide): a face flux (2^60, near: 2^61), a viscous flux (2^58, 2^59) or a sum
+// (2^61: the weighted sums of three directions stay below 2^63).  States at the corners of the range bring
+// the sums to 0.8 of 2^63, and one that wrapped would still be seen, being below 1.75 of it.  need[] takes the bits by which
+// fluxes pass (kMxT, kMxH: momentum, energy); a sum that passes takes two of each.  check: only the fluxes.
 // Viscous part: omega_i (D f + lifting)_i = sum_{j != i} Q_ij f_j + f_next/2 (i = p) - f_prev/2
 // (i = 0), the diagonal of D cancelling the lifting's interior half (fv: planes of this direction,
 // plane stride N; v_hi, v_lo: nodes whose values stand for f_next and f_prev).
 template <int P1, int TIER, bool NS, int DIRS>
-__device__ __forceinline__ bool volume_line_fx(const FxParams& P, const FxScale& sc, int m, int a, int b, fx wm,
+__device__ __forceinline__ int volume_line_fx(const FxParams& P, const FxScale& sc, int m, int a, int b, fx wm,
                                                const fx* __restrict__ z, const float4* __restrict__ zf,
                                                const double* __restrict__ f_hi, const double* __restrict__ f_lo,
                                                long long fs, const double* __restrict__ fv, long long g0,
                                                long long v_hi, long long v_lo, long long N, fx* __restrict__ acc,
-                                               int stride) {
+                                               int stride, int* __restrict__ need, int need_stride, bool check) {
   const int c1 = m, c2 = m == 2 ? 0 : m + 1, c3 = m == 0 ? 2 : m - 1;
   const int comp[5] = {0, (1 + c1) * stride, (1 + c2) * stride, (1 + c3) * stride, 4 * stride};
   fx r[P1][5];
@@ -160,7 +163,7 @@ __device__ __forceinline__ bool volume_line_fx(const FxParams& P, const FxScale&
   for (int i = 0; i < P1; ++i)
 #pragma unroll
     for (int c = 0; c < 5; ++c) r[i][c] = 0;
-  bool fits = true;
+  int mass = 0, mom = 0, ener = 0;  // bits beyond the scales (0 or less: fits)
   {
     const int v[5] = {0, 1 + c1, 1 + c2, 1 + c3, 4};
 #pragma unroll
@@ -168,7 +171,8 @@ __device__ __forceinline__ bool volume_line_fx(const FxParams& P, const FxScale&
       const int emax = 1084 + fx_unit(sc, c == 0 ? 0 : (c == 4 ? 4 : 1));
       const double hi = f_hi[v[c] * fs], lo = f_lo[v[c] * fs];
       const int top = max(__double2hiint(hi) & 0x7fffffff, __double2hiint(lo) & 0x7fffffff) >> 20;
-      fits &= top <= emax - (TIER == kFxNear ? 1 : 2);
+      int& over = c == 0 ? mass : (c == 4 ? ener : mom);
+      over = max(over, top - (emax - (TIER == kFxNear ? 1 : 2)));
       r[P1 - 1][c] = fx_from_double(hi, emax);
       r[0][c] = -fx_from_double(lo, emax);
     }
@@ -188,7 +192,8 @@ __device__ __forceinline__ bool volume_line_fx(const FxParams& P, const FxScale&
           top = max(top, __double2hiint(fl[j]) & 0x7fffffff);
           n[j] = fx_from_double(fl[j], emax);
         }
-        fits &= (top >> 20) <= emax - (TIER == kFxNear ? 2 : 3);
+        int& over = c == 4 ? ener : mom;
+        over = max(over, (top >> 20) - (emax - (TIER == kFxNear ? 2 : 3)));
         r[P1 - 1][c] -= fx_from_double(hi, emax) >> 2;
         r[0][c] += fx_from_double(lo, emax) >> 2;
 #pragma unroll
@@ -203,7 +208,12 @@ __device__ __forceinline__ bool volume_line_fx(const FxParams& P, const FxScale&
   }
   // the element is done again in other scales, or in FP64: no pair of this line is formed (viscous
   // shock p = 3 25^3, where a band of elements needs the second attempt: 744 -> 693 us per launch)
-  if (!fits) return false;
+  if ((mass | mom | ener) > 0) {
+    atomicMax(need + kMxT * need_stride, mom);
+    atomicMax(need + kMxH * need_stride, ener);
+    return mass > 0 ? kFxMass : kFxWide;
+  }
+  if (check) return 0;
 #pragma unroll
   for (int i = 0; i < P1 - 1; ++i) {
     fx si[5];
@@ -243,7 +253,10 @@ __device__ __forceinline__ bool volume_line_fx(const FxParams& P, const FxScale&
         acc[comp[c] + n] = m == 0 ? val : acc[comp[c] + n] + val;
     }
   }
-  return !(over & 0xc0000000);
+  if (!(over & 0xc0000000)) return 0;
+  atomicMax(need + kMxT * need_stride, 2);
+  atomicMax(need + kMxH * need_stride, 2);
+  return kFxWide;
 }
 
 // Tiles (elements per CTA, threads) and register bounds, measured on GB300 (one right-hand side,
@@ -332,11 +345,13 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
     if (threadIdx.x < nel) {
       const int el = threadIdx.x;
       scale[el] = fx_scale(meta[kMx1 * EPB + el], meta[kMn1 * EPB + el], meta[kMx5 * EPB + el],
-                           meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt, NS ? kFxViscous : kFxFine);
+                           meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt);
+      // (heat conduction does not vanish with the velocity)
+      if constexpr (NS) scale[el].se = min(max(1018 - scale[el].ev, 0), kFxMargin);
       if constexpr (NS) viscous = fx_viscous_element(P, scale[el], fx_metric_exponent(geom_of(P, inst_of(P, e0 + el))));
     }
-    // Where the viscous fluxes may not fit: looked at before any pair is formed, and the second
-    // attempt's scales at once if they do not (one that does not fit all the same is found below).
+    // Where the viscous fluxes may not fit: looked at before any pair is formed, and the room they need
+    // given at once (an element that does not fit all the same is found below).
     // Viscous shock 25^3 p = 3 693 -> 540 us per launch; looked at without the estimate before it, Navier--
     // Stokes p = 4 takes 941 us (930 with, 924 with neither).
     if constexpr (NS) {
@@ -358,10 +373,9 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
         __syncthreads();
         if (threadIdx.x < nel) {
           const int el = threadIdx.x, room = scale[el].tier == kFxNear ? 1081 : 1080;  // volume_line_fx's limits
-          if ((meta[kMxT * EPB + el] >> 20) > room + fx_unit(scale[el], 1) ||
-              (meta[kMxH * EPB + el] >> 20) > room + fx_unit(scale[el], 4))
-            scale[el] = fx_scale(meta[kMx1 * EPB + el], meta[kMn1 * EPB + el], meta[kMx5 * EPB + el],
-                                 meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt, kFxCoarse);
+          int &t = meta[kMxT * EPB + el], &h = meta[kMxH * EPB + el];
+          fx_widen(scale[el], max((t >> 20) - room - fx_unit(scale[el], 1), 0), max((h >> 20) - room - fx_unit(scale[el], 4), 0));
+          t = h = 0;
         }
       }
     }
@@ -403,7 +417,8 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
         const int el = l / P2, ab = l % P2, e = e0 + el;
         const FxScale& sc = scale[el];
         if (sc.tier == kFxSlow || (attempt && !meta[kRetry * EPB + el])) continue;
-        if (DIRS == 1 && m && meta[kBad * EPB + el]) continue;  // (set in an earlier direction)
+        // (passed in an earlier direction: only how far this one's fluxes pass)
+        const bool check = DIRS == 1 && m && meta[kBad * EPB + el];
         const InstGeom& G = geom_of(P, inst_of(P, e));
         const int em = fx_metric_exponent(G);
         const fx wm = fx_from_double(G.metric[m], em);
@@ -422,21 +437,21 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
                       : (long long)neighbour(P, e, m, -1) * Np + line_node<P1>(m, a, b, P1 - 1);
         }
         const double* fv = NS ? fV + (long long)(m * 4) * N : nullptr;
-        bool fits;
+        int beyond;
         if (sc.tier == kFxNear)
-          fits = volume_line_fx<P1, kFxNear, NS, DIRS>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs, fv, g0,
-                                                 v_hi, v_lo, N, acc + el * Np, ST);
+          beyond = volume_line_fx<P1, kFxNear, NS, DIRS>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs, fv, g0,
+                                                 v_hi, v_lo, N, acc + el * Np, ST, meta + el, EPB, check);
         else
-          fits = volume_line_fx<P1, kFxFar, NS, DIRS>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs, fv, g0,
-                                                v_hi, v_lo, N, acc + el * Np, ST);
-        if (!fits) meta[kBad * EPB + el] = 1;
+          beyond = volume_line_fx<P1, kFxFar, NS, DIRS>(P, sc, m, a, b, wm, z + el * Np, zf + el * Np, f_hi, f_lo, fs, fv, g0,
+                                                v_hi, v_lo, N, acc + el * Np, ST, meta + el, EPB, check);
+        if (beyond) atomicOr(meta + kBad * EPB + el, beyond);
       }
       __syncthreads();
     }
     const bool bad = my < nel && scale[my].tier != kFxSlow && meta[kBad * EPB + my];
     if (attempt == 0 && bad) {
-      scale[my] = fx_scale(meta[kMx1 * EPB + my], meta[kMn1 * EPB + my], meta[kMx5 * EPB + my], meta[kMn5 * EPB + my],
-                           meta[kMxV * EPB + my], P.fxC, P.fxKt, kFxCoarse);
+      fx_widen(scale[my], meta[kMxT * EPB + my], meta[kMxH * EPB + my]);
+      if (meta[kBad * EPB + my] & kFxMass) scale[my].tier = kFxSlow;
       meta[kRetry * EPB + my] = 1;
       meta[kBad * EPB + my] = 0;
     }

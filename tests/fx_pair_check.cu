@@ -1,5 +1,6 @@
 // Host check of the fixed-point two-point flux (csrc/es_fx.cuh) at the edges of its range.
 //   slow  gas slower than the velocities' other scales: mass and energy flux relative to themselves
+//   room  the room that fluxes beyond an element's scales are given
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -101,5 +102,30 @@ int main(int argc, char** argv) {
           }
           printf("slow %g %g %g out %d mass %.2Lf energy %.2Lf\n", gam, speed, var, out, ldexpl(mass, 53), ldexpl(energy, 53));
         }
+  if (!strcmp(argv[1], "room")) {
+    int wrong = 0, fp64 = 0, taken = 0;
+    for (int Ev = -29; Ev <= 2; ++Ev)
+      for (int first = 0; first < 6; ++first)
+        for (int dm = 0; dm < 12; ++dm)
+          for (int de = 0; de < 45; ++de) {
+            const int one = 1023 << 20, mxv = (1022 + Ev) << 20;  // z1 = z5 = 1, |z_v| = 2^(Ev - 1)
+            FxScale a = fx_scale(one, one, one, one, mxv - (1 << 20) + 1, fx(3) << 60, 4);
+            if (a.tier == kFxSlow) continue;
+            a.se += first;
+            FxScale b = a;
+            fx_widen(b, dm, de);
+            const int um = fx_unit(b, 1) - fx_unit(a, 1), ue = fx_unit(b, 4) - fx_unit(a, 4);
+            const bool fits = dm <= 6 && first + de <= std::max(-(a.ev - 1022), 0) + 6;
+            if (b.tier == kFxSlow) {
+              ++fp64;
+              wrong += fits;
+            } else {
+              ++taken;
+              wrong += !fits || um < dm || ue < de || um > (dm ? dm + 3 : 0) || ue > (de ? de + 3 : 0);
+            }
+            wrong += b.sv < 0 || b.sv > 63 || b.se < 0 || b.se > 63;
+          }
+    printf("room wrong %d taken %d fp64 %d\n", wrong, taken, fp64);
+  }
   return 0;
 }

@@ -4,6 +4,8 @@ Bounds.
 * Slow gas: the factors of mass and energy flux carry units of 2^-62 of the block scale, 64 of them in all
   (tests/test_fx_flux.py); with |Q_ij| >= 1/4, velocity and z5 at least half of their blocks' the mass flux is above
   2^-4 of the scale and the energy flux above 2^-6, so 64 units are 2 and 8 units of 2^-53 of the flux itself.
+* Room beyond an element's scales: no more than three bits above what its fluxes need, of the five that the sums
+  have over a double's.
 """
 import os
 import shutil
@@ -36,3 +38,9 @@ def test_slow_gas(check):
     for ln in rows:
         assert int(ln[5]) == 0, ln
         assert float(ln[7]) <= 2.0 and float(ln[9]) <= 8.0, ln
+
+
+def test_room_for_larger_fluxes(check):
+    # what the fluxes need and three bits beside it, up to 2^6 times the pressure and the enthalpy flux at sound speed
+    (row,) = check("room")
+    assert int(row[2]) == 0 and int(row[4]) > 1000 and int(row[6]) > 1000, row
