@@ -180,9 +180,12 @@ ES_HD fx fx_rcp(fx s, float q) {
 // (F(u) = atanh(sqrt u)/sqrt u), with 64 fractional bits.
 // kFxNear, |r| <= 0.01: three terms (truncation below 1.2e-17, as in the FP64 flux) on the FP32
 // pipe, which the integer products leave idle: a and b as pairs of floats (23 + 24 bits of the
-// block fraction, so that sum and difference of the upper parts are exact), r and u as pairs,
-// relative error below 2^-40; the correction is below 3.4e-5, so its absolute error is below
-// 2^-54.  The pair becomes an integer through two additions to powers of two.
+// block fraction, so that sum and difference of the upper parts are exact), r and u as pairs.  At the
+// limit the dropped bits of a and b move r by up to 2^-46 and the correction by 2/3 |r| of it, 0.9 units
+// of 2^-53, the FP32 roundings of the u^2 term (below 2^-28.9) by 2.6 and those of its sum by 1.5: five at
+// most, 4.0 measured, and 0.6 at |r| = 0.005.  The flux is still closer than in FP64, whose every product rounds: up to
+// the limit 0.17 units of itself in the mass and 0.4 in the energy on average (FP64: 1.0 and 2.1), 1.9 and 3.3 at
+// worst (5.6 and 11).  The pair becomes an integer through two additions to powers of two.
 // kFxFar, |r| <= 0.2: twelve terms in fixed point (truncation below 2^-59; the terms from u^6 on
 // enter with a weight below 2^-23 and are summed in 32 bits); r with 61 fractional bits.
 constexpr int kFxSlow = 0, kFxNear = 1, kFxFar = 2;

@@ -1,6 +1,7 @@
 // Host check of the fixed-point two-point flux (csrc/es_fx.cuh) at the edges of its range.
 //   slow  gas slower than the velocities' other scales: mass and energy flux relative to themselves
 //   room  the room that fluxes beyond an element's scales are given
+//   near  the logarithmic-mean correction and the flux up to the limit of the near tier
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -29,6 +30,19 @@ static void flux(const double* p, const double* q, L gam, L f[5]) {  // z1, z_m,
   f[2] = m * v;
   f[3] = m * w;
   f[4] = u * gam / (gam - 1) * p1 * ((gam + 1) / (2 * gam) * g * f1 + (gam - 1) / (2 * gam)) + m * (u * u + v * v + w * w) / 2;
+}
+
+// the FP64 kernels' form of it
+static void flux_double(const double* a, const double* b, double g, double f[5]) {
+  const double S1 = a[0] + b[0], S5 = a[4] + b[4], P15 = S1 * S5, inv = 1 / P15, inv1 = S5 * inv;
+  const double r1 = (a[0] - b[0]) * inv1, r5 = (a[4] - b[4]) * (S1 * inv), u1 = r1 * r1, u5 = r5 * r5;
+  const double f1 = 1 + u1 * (1.0 / 3 + u1 * (1.0 / 5 + u1 * (1.0 / 7)));
+  const double g5 = 0.25 - u5 * (1.0 / 12 + u5 * (1.0 / 45 + u5 * (11.0 / 945)));
+  const double rho = P15 * g5, u = (a[1] + b[1]) * inv1, v = (a[2] + b[2]) * inv1, w = (a[3] + b[3]) * inv1;
+  const double p1 = S5 * inv1, mass = rho * u;
+  const double p2 = p1 * (2 * (g + 1) / (g - 1) * (g5 * f1) + 0.5);
+  f[0] = mass;
+  f[4] = u * p2 + 0.5 * mass * (u * u + v * v + w * w);
 }
 
 struct Gas {
@@ -126,6 +140,55 @@ int main(int argc, char** argv) {
             wrong += b.sv < 0 || b.sv > 63 || b.se < 0 || b.se > 63;
           }
     printf("room wrong %d taken %d fp64 %d\n", wrong, taken, fp64);
+  }
+  if (!strcmp(argv[1], "near")) {
+    // the correction alone, |r| up to 0.0101 by steps; the tier that the pair's high words give
+    L worst = 0;
+    int near = 0;
+    for (int it = 0; it < 3000000; ++it) {
+      const double r = 0.0101 * (it % 3 ? U(R) : (1 - 1e-3 * fabs(U(R))) * 0.5), b = it % 5 ? 1 + fabs(U(R)) : 2 - 1e-3 * fabs(U(R)), a = b * (1 + r) / (1 - r);
+      const FxScale t = fx_scale(fx_hi_word(std::max(a, b)), fx_hi_word(std::min(a, b)), 1023 << 20, 1023 << 20, 1020 << 20, fx(3) << 60, 4);
+      if (t.tier != kFxNear) continue;
+      ++near;
+      const FxPair x = fx_pair(fx_from_positive(a, t.e1)), y = fx_pair(fx_from_positive(b, t.e1));
+      const float q = fx_rcpf(x.h + y.h);
+      const L rr = ((L)a - b) / ((L)a + b), f = series(rr);
+      worst = std::max(worst, fabsl(ldexpl((L)fx_near(x, y, q, 0.2f, 1.0f / 7.0f), -64) - (f - 1)));
+      worst = std::max(worst, fabsl(ldexpl((L)fx_near(x, y, q, 4.0f / 45.0f, 44.0f / 945.0f), -64) - (1 - 1 / f)));
+    }
+    printf("correction %d units %.3Lf\n", near, ldexpl(worst, 53));
+    // the flux relative to itself, and the FP64 formula's
+    for (double gam : {1.4, 5.0 / 3.0, 1.1, 4.0})
+      for (double mach : {1e-3, 0.3, 1.2, 3.0}) {
+        const Gas gas(gam);
+        L mean[2][2] = {}, most[2][2] = {};
+        int n = 0;
+        for (int it = 0; it < 60000; ++it) {
+          double z[2][5], f[5];
+          const double z1 = exp(6 * U(R)), z5 = exp(6 * U(R)), r = 0.0099 * (it % 2 ? 1 : fabs(U(R)));
+          for (int i = 0; i < 2; ++i) {
+            z[i][0] = z1 * (i ? (1 - r) / (1 + r) : 1);
+            z[i][4] = z5 * (i ? 1 : (1 - r) / (1 + r));
+            for (int k = 1; k < 4; ++k) z[i][k] = mach * (0.3 + 0.3 * fabs(U(R)));
+          }
+          if (!pair(z[0], z[1], gam, gas, 1ll << 62, diff, want, s) || s.tier != kFxNear) continue;
+          flux_double(z[0], z[1], gam, f);
+          ++n;
+          for (int v : {0, 4}) {
+            const L e[2] = {(diff[v] + ldexpl(fabsl(want[v]), -53)) / fabsl(want[v]), fabsl(f[v] / want[v] - 1)};
+            for (int k = 0; k < 2; ++k) {
+              mean[v / 4][k] += e[k];
+              most[v / 4][k] = std::max(most[v / 4][k], e[k]);
+            }
+          }
+        }
+        printf("near %g %g pairs %d", gam, mach, n);
+        for (auto& m : mean)
+          for (L x : m) printf(" %.2Lf", ldexpl(x / n, 53));
+        for (auto& m : most)
+          for (L x : m) printf(" %.2Lf", ldexpl(x, 53));
+        puts("");
+      }
   }
   return 0;
 }

@@ -6,6 +6,9 @@ Bounds.
   2^-4 of the scale and the energy flux above 2^-6, so 64 units are 2 and 8 units of 2^-53 of the flux itself.
 * Room beyond an element's scales: no more than three bits above what its fluxes need, of the five that the sums
   have over a double's.
+* Near tier: the correction is good to five units of 2^-53 at its limit (the sum of its roundings stands beside it
+  in the header), and the flux is no further from long double than the FP64 kernels' form of it, on average and
+  at worst.
 """
 import os
 import shutil
@@ -44,3 +47,15 @@ def test_room_for_larger_fluxes(check):
     # what the fluxes need and three bits beside it, up to 2^6 times the pressure and the enthalpy flux at sound speed
     (row,) = check("room")
     assert int(row[2]) == 0 and int(row[4]) > 1000 and int(row[6]) > 1000, row
+
+
+def test_near_tier_to_its_limit(check):
+    rows = check("near")
+    assert rows[0][0] == "correction" and int(rows[0][1]) > 100000
+    assert float(rows[0][3]) <= 5.0, rows[0]
+    assert len(rows) == 1 + 4 * 4
+    for ln in rows[1:]:
+        assert int(ln[4]) > 10000, ln
+        values = list(map(float, ln[5:13]))  # mean mass, energy; largest mass, energy: fixed point, FP64
+        for fixed, double in zip(values[::2], values[1::2]):
+            assert fixed <= double, ln
