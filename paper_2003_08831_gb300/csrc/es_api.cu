@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "../../include/es.h"
+#include "es_fx.cuh"
 #include "es_launch.h"
 
 using namespace es;
@@ -254,6 +255,7 @@ void build_params(const es_config& C, FxParams* out) {
   P.ff_est = (C.precision == ES_MIXED_FF || C.precision == ES_FP64X) ? 1 : 0;
   P.visc_pen = C.mu > 0.0 ? C.visc_diss : 0.0;
   P.g0 = instance_geom(C, 0);
+  P.fxIso = fx_metrics_close(P.g0.metric);
   P.geom = nullptr;
   P.elem_inst = nullptr;
 }
@@ -565,6 +567,7 @@ int group_init(Group& g, const es_config* insts, int n, int stages, bool own_sta
   g.geom.resize(n);
   for (int i = 0; i < n; ++i) {
     g.geom[i] = instance_geom(insts[i], (int)K);
+    g.P.fxIso &= fx_metrics_close(g.geom[i].metric);
     K += (long long)insts[i].nx * insts[i].ny * insts[i].nz;
   }
   if (K > (1LL << 30)) return ES_ERR_INVALID;

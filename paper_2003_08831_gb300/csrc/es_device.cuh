@@ -90,6 +90,7 @@ struct FxParams : Params {
   long long fxG;                   // gam - 1 = fxG 2^(fxEg - 63), 2^62 <= fxG < 2^63
   long long fxI;                   // 1/(gam - 1) = fxI 2^(fxEi - 62), 2^61 <= fxI < 2^62
   int fxKt, fxKw, fxEg, fxEi;
+  int fxIso;                       // fx_metrics_close of every instance
 };
 
 template <typename T> __device__ __forceinline__ const FluxConst<T>& flux_const(const Params& P);

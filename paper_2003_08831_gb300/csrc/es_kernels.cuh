@@ -372,6 +372,11 @@ __device__ __forceinline__ bool stage_z_ff(const Params& P, const ff uf[5], cons
 }
 
 // ---------------------------------------------------------------------------
+// whether an instance's metrics allow the fixed-point forms
+__device__ __forceinline__ bool fx_mesh(const FxParams& P, int inst) {
+  return P.fxIso || fx_metrics_close(geom_of(P, inst).metric);
+}
+
 // FP64 forms of the stage preparation's pieces for states outside the fixed-point range
 // (es_prep_fx.cuh), out of line: they are rare and would cost the common path its registers.
 static __device__ __noinline__ bool param_vector_fp64(const double* y, double gam, double* z) {
@@ -486,7 +491,7 @@ __device__ __forceinline__ void prep_body(const PrepParams<FP64>& P, const Stage
       if (planes) {
         double z[6];
         FxState zy;
-        if (ok) {
+        if (ok && fx_mesh(P, inst)) {
           fx_parameters(b, P.fxG, P.fxEg, zy);
           fx_state_planes(zy, z);
         } else if (!param_vector_fp64(y, gam, z)) {
@@ -617,7 +622,12 @@ __device__ __forceinline__ void face_flux(const Zstate<TF>& L, TF izL, const Zst
     z_to_q(R, izR, C, qR, lR, m);
     const TF lam = TF(0.5) * fmax(lL, lR);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) f[v] -= lam * (qR[v] - qL[v]);
+    for (int v = 0; v < 5; ++v) {
+      // (FP64: a product contracted into the difference would leave its rounding as a jump between equal
+      // states, which a thin element's metric multiplies)
+      if constexpr (std::is_same<TF, double>::value) f[v] -= lam * __dadd_rn(qR[v], -qL[v]);
+      else f[v] -= lam * (qR[v] - qL[v]);
+    }
   }
 }
 
@@ -680,11 +690,12 @@ static __device__ __noinline__ void face_flux_fp64(const Zstate<double>& L, doub
 template <typename TF> using FaceParams = std::conditional_t<std::is_same<TF, double>::value, FxParams, Params>;
 // face_flux with k_face's constants: in FP64 mode through the fixed-point form (es_face_fx.cuh),
 // the matrix dissipation always in FP64
-template <typename TF>
-__device__ __forceinline__ void interface_flux(const FaceParams<TF>& P, const FluxConst<TF>& C, const Zstate<TF>& L, TF izL,
+// (ISO: every instance's metrics allow the fixed-point form)
+template <typename TF, bool ISO>
+__device__ __forceinline__ void interface_flux(const FaceParams<TF>& P, int e, const FluxConst<TF>& C, const Zstate<TF>& L, TF izL,
                                                const Zstate<TF>& R, TF izR, int m, TF f[5]) {
   if constexpr (std::is_same<TF, double>::value) {
-    if (fx_face_flux(L.z, R.z, m, P.fxC, P.fxKt, C.sqrt_gam, P.diss, f)) {
+    if ((ISO || fx_mesh(P, inst_of(P, e))) && fx_face_flux(L.z, R.z, m, P.fxC, P.fxKt, C.sqrt_gam, P.diss, f)) {
       if (P.diss == 2) matrix_dissipation(L, R, m, C, f);
     } else {
       face_flux_fp64(L, izL, R, izR, m, C, P.diss, f);
@@ -696,7 +707,7 @@ __device__ __forceinline__ void interface_flux(const FaceParams<TF>& P, const Fl
 
 // VPEN: with the diss^V penalty (a separate instantiation keeps the common path's
 // register count)
-template <int P1, typename TF, bool VPEN>
+template <int P1, typename TF, bool VPEN, bool ISO>
 __device__ __forceinline__ void face_node(const FaceParams<TF>& P, const FluxConst<TF>& C, const TF* __restrict__ aux,
                                           TF* __restrict__ F, TF* __restrict__ FL, int e, int m, int ab) {
   constexpr int P2 = P1 * P1, Np = P1 * P2;
@@ -715,7 +726,7 @@ __device__ __forceinline__ void face_node(const FaceParams<TF>& P, const FluxCon
     izR = aux[5 * N + gR];
   }
   TF f[5];
-  interface_flux(P, C, L, izL, R, izR, m, f);
+  interface_flux<TF, ISO>(P, e, C, L, izL, R, izR, m, f);
   // diss^V penalty scale alpha (2/h_m)(1/omega_0)
   TF sig = TF(0);
   if constexpr (VPEN) {
@@ -730,7 +741,7 @@ __device__ __forceinline__ void face_node(const FaceParams<TF>& P, const FluxCon
     const long long g0 = (long long)e * Np + line_node<P1>(m, a, b, 0);
     const Zstate<TF> I = load_z<P1, TF>(aux, N, g0);
     const TF izI = aux[5 * N + g0];
-    interface_flux(P, C, B, izB, I, izI, m, f);
+    interface_flux<TF, ISO>(P, e, C, B, izB, I, izI, m, f);
     if constexpr (VPEN) visc_penalty(B, izB, I, izI, m, sig, P, f);
 #pragma unroll
     for (int v = 0; v < 5; ++v) FL[((long long)(m * 5 + v) * P.K + e) * P2 + ab] = f[v];
@@ -745,21 +756,21 @@ __global__ void k_face(Params P, const TF* __restrict__ aux, TF* __restrict__ F,
        idx += (long long)gridDim.x * blockDim.x) {
     const int m = int(idx / ((long long)P.K * P2));
     const long long rem = idx - (long long)m * P.K * P2;
-    face_node<P1, TF, VPEN>(P, C, aux, F, FL, int(rem / P2), m, int(rem % P2));
+    face_node<P1, TF, VPEN, true>(P, C, aux, F, FL, int(rem / P2), m, int(rem % P2));
   }
 }
 // FP64: one direction per blockIdx.y and one face node per thread (no 64-bit divisions), 80
 // registers for three blocks of 256 threads per SM (two at 114): the kernel waits for its loads and
 // its dependent products.  Taylor--Green 32^3 p = 3 119 -> 102 us per launch, Navier--Stokes p = 4
 // 193 -> 162 us.  The other precisions keep the loop (float-float: 70 us; 84 in this form).
-template <int P1, bool VPEN>
+template <int P1, bool VPEN, bool ISO>
 __global__ void __launch_bounds__(256, 3) k_face_fp64(const __grid_constant__ FxParams P, const double* __restrict__ aux,
                                                       double* __restrict__ F, double* __restrict__ FL) {
   constexpr unsigned P2 = P1 * P1;
   // (below 2^32 face nodes per direction: 2^32 are 700 GB of states)
   const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < unsigned(P.K) * P2)
-    face_node<P1, double, VPEN>(P, P.Cd, aux, F, FL, int(idx / P2), blockIdx.y, int(idx % P2));
+    face_node<P1, double, VPEN, ISO>(P, P.Cd, aux, F, FL, int(idx / P2), blockIdx.y, int(idx % P2));
 }
 
 // ---------------------------------------------------------------------------
@@ -1978,8 +1989,9 @@ void Launcher<P1, TF>::face(const FxParams& P, const void* aux, void* F, void* F
   TF *f = static_cast<TF*>(F), *fl = static_cast<TF*>(FL);
   if constexpr (std::is_same<TF, double>::value) {
     const dim3 blocks((unsigned(P.K) * (P1 * P1) + nb - 1) / nb, 3);
-    if (P.visc_pen > 0.0) k_face_fp64<P1, true><<<blocks, nb, 0, st>>>(P, a, f, fl);
-    else k_face_fp64<P1, false><<<blocks, nb, 0, st>>>(P, a, f, fl);
+    const auto k = P.fxIso ? (P.visc_pen > 0.0 ? k_face_fp64<P1, true, true> : k_face_fp64<P1, false, true>)
+                           : (P.visc_pen > 0.0 ? k_face_fp64<P1, true, false> : k_face_fp64<P1, false, false>);
+    k<<<blocks, nb, 0, st>>>(P, a, f, fl);
   } else {
     if (P.visc_pen > 0.0) k_face<P1, TF, true><<<grid, nb, 0, st>>>(P, a, f, fl);
     else k_face<P1, TF, false><<<grid, nb, 0, st>>>(P, a, f, fl);

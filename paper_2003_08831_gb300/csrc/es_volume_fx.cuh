@@ -346,6 +346,7 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
       const int el = threadIdx.x;
       scale[el] = fx_scale(meta[kMx1 * EPB + el], meta[kMn1 * EPB + el], meta[kMx5 * EPB + el],
                            meta[kMn5 * EPB + el], meta[kMxV * EPB + el], P.fxC, P.fxKt);
+      if (!fx_mesh(P, inst_of(P, e0 + el))) scale[el].tier = kFxSlow;
       // (heat conduction does not vanish with the velocity)
       if constexpr (NS) scale[el].se = min(max(1018 - scale[el].ev, 0), kFxMargin);
       if constexpr (NS) viscous = fx_viscous_element(P, scale[el], fx_metric_exponent(geom_of(P, inst_of(P, e0 + el))));

@@ -2,6 +2,7 @@
 //   slow  gas slower than the velocities' other scales: mass and energy flux relative to themselves
 //   room  the room that fluxes beyond an element's scales are given
 //   near  the logarithmic-mean correction and the flux up to the limit of the near tier
+//   metrics  rates of an element with anisotropic metrics, flow along the coarse direction
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -82,6 +83,67 @@ static bool pair(const double a[5], const double b[5], double gam, const Gas& ga
     diff[v] = fabsl(ldexpl((L)g[v], fx_unit(s, v)) - want[v]) - ldexpl(fabsl(want[v]), -53);
   }
   return true;
+}
+
+// LGL nodes, and per degree Q_ij = omega_i D_ij, 1/omega_i
+struct Line {
+  int n;
+  L x[6], w[6], Q[6][6];
+  explicit Line(int p) : n(p + 1) {
+    L P[6];
+    for (int i = 0; i < n; ++i) {
+      x[i] = -cosl(3.14159265358979323846264338327950288L * i / p);
+      for (int it = 0; it < 60; ++it) {
+        L a = 1, b = x[i];
+        for (int k = 1; k < p; ++k) {
+          const L c = ((2 * k + 1) * x[i] * b - k * a) / (k + 1);
+          a = b;
+          b = c;
+        }
+        P[i] = b;
+        if (i > 0 && i < p) x[i] += (a - x[i] * b) / ((p + 1) * b);
+      }
+      w[i] = 2 / (p * (p + 1) * P[i] * P[i]);
+    }
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j) Q[i][j] = i == j ? 0 : w[i] * P[i] / (P[j] * (x[i] - x[j]));
+  }
+  fx q(int i, int j) const { return i == j ? 0 : llrintl(ldexpl(Q[i][j], 63)); }
+};
+
+// the line sums of n nodes (component order z1, z_m, the others, z5), exact
+static void line_sums(const Line& l, const double (*z)[5], const FxScale& s, __int128 r[6][5]) {
+  fx x[6][5];
+  FxPair p[6][2];
+  for (int i = 0; i < l.n; ++i) {
+    x[i][0] = fx_from_positive(z[i][0], s.e1);
+    x[i][4] = fx_from_positive(z[i][4], s.e5);
+    for (int k = 1; k < 4; ++k) x[i][k] = fx_from_double(z[i][k], s.ev);
+    p[i][0] = fx_pair(x[i][0]);
+    p[i][1] = fx_pair(x[i][4]);
+    for (int c = 0; c < 5; ++c) r[i][c] = 0;
+  }
+  for (int i = 0; i < l.n; ++i)
+    for (int j = i + 1; j < l.n; ++j) {
+      fx g[5];
+      if (s.tier == kFxNear) fx_flux<kFxNear>(x[i], p[i], x[j], p[j], l.q(i, j), s, g);
+      else fx_flux<kFxFar>(x[i], p[i], x[j], p[j], l.q(i, j), s, g);
+      for (int c = 0; c < 5; ++c) {
+        r[i][c] += g[c];
+        r[j][c] -= g[c];
+      }
+    }
+}
+static FxScale scale(const double (*z)[5], int n, const Gas& gas) {
+  int mx1 = 0, mn1 = 0x7fffffff, mx5 = 0, mn5 = 0x7fffffff, mxv = 0;
+  for (int i = 0; i < n; ++i) {
+    mx1 = std::max(mx1, fx_hi_word(z[i][0]));
+    mn1 = std::min(mn1, fx_hi_word(z[i][0]));
+    mx5 = std::max(mx5, fx_hi_word(z[i][4]));
+    mn5 = std::min(mn5, fx_hi_word(z[i][4]));
+    for (int k = 1; k < 4; ++k) mxv = std::max(mxv, fx_hi_word(z[i][k]) & 0x7fffffff);
+  }
+  return fx_scale(mx1, mn1, mx5, mn5, mxv, gas.C1, gas.kt);
 }
 
 int main(int argc, char** argv) {
@@ -190,5 +252,55 @@ int main(int argc, char** argv) {
         puts("");
       }
   }
+  if (!strcmp(argv[1], "metrics"))
+    for (int p = 2; p <= 5; ++p)
+      for (double ratio : {1.0, 3.9, 7.9, 15.9, 16.5, 17.5, 33.0, 1e3}) {
+        // sums of the coarse direction, as the kernel joins them: r (1/omega) metric in units of the largest metric
+        const Line l(p);
+        const Gas gas(1.4);
+        const double metric[3] = {1.9, 1.9 * ratio, 1.9 * ratio};
+        L err[5] = {}, err64[5] = {}, top[5] = {};
+        for (int it = 0; it < 300; ++it) {
+          double z[6][5];
+          const double a = 3 * U(R);
+          for (int i = 0; i <= p; ++i) {
+            const double x = (double)l.x[i];
+            z[i][0] = 1.1 + 0.01 * sin(x + a);
+            z[i][4] = 1.3 + 0.01 * cos(x - a);
+            z[i][1] = 0.3 + 0.1 * sin(x + 2 * a);
+            z[i][2] = 0.2 * cos(x + a);
+            z[i][3] = 0;
+          }
+          const FxScale t = scale(z, p + 1, gas);
+          __int128 r[6][5];
+          line_sums(l, z, t, r);
+          const int em = (fx_hi_word(metric[1])) >> 20;
+          int kw = 0;
+          while ((1 << kw) <= p * (p + 1) / 2) ++kw;
+          for (int i = 0; i <= p; ++i) {
+            const fx w = fx_mul63(llrintl(ldexpl(1 / l.w[i], 63 - kw)), fx_from_double(metric[0], em));
+            L k[5] = {}, f[5];
+            double k64[5] = {};
+            for (int j = 0; j <= p; ++j) {
+              if (j == i) continue;
+              flux(z[i], z[j], 1.4, f);
+              const double d = (double)(2 * l.Q[i][j] / l.w[i]);
+              for (int c = 0; c < 5; ++c) {
+                k[c] += 2 * l.Q[i][j] / l.w[i] * metric[0] * f[c];
+                k64[c] = fma(d, (double)f[c], k64[c]);
+              }
+            }
+            for (int c = 0; c < 5; ++c) {
+              const L got = ldexpl((L)fx_mul63(fx(r[i][c]), w), fx_unit(t, c) + em - 1022 + kw + 1);
+              top[c] = std::max(top[c], fabsl(k[c]));
+              err[c] = std::max(err[c], fabsl(got - k[c]));
+              err64[c] = std::max(err64[c], fabsl(metric[0] * k64[c] - k[c]));
+            }
+          }
+        }
+        printf("metrics %d %g taken %d", p, ratio, fx_metrics_close(metric));
+        for (int c : {0, 1, 4}) printf(" %.2Le %.2Le", err[c] / top[c], err64[c] / top[c]);
+        puts("");
+      }
   return 0;
 }

@@ -9,6 +9,7 @@ Bounds.
 * Near tier: the correction is good to five units of 2^-53 at its limit (the sum of its roundings stands beside it
   in the header), and the flux is no further from long double than the FP64 kernels' form of it, on average and
   at worst.
+* Metrics: where they are taken, the sums are no further off than the same sums in FP64.
 """
 import os
 import shutil
@@ -59,3 +60,14 @@ def test_near_tier_to_its_limit(check):
         values = list(map(float, ln[5:13]))  # mean mass, energy; largest mass, energy: fixed point, FP64
         for fixed, double in zip(values[::2], values[1::2]):
             assert fixed <= double, ln
+
+
+def test_metrics(check):
+    rows = check("metrics")
+    assert len(rows) == 4 * 8
+    for ln in rows:
+        taken, ratio = int(ln[4]), float(ln[2])
+        assert taken == (ratio < 17.0), ln  # 1.9 and 1.9 ratio: exponents up to four apart
+        if taken:
+            for fixed, double in zip(ln[5::2], ln[6::2]):
+                assert float(fixed) <= float(double), ln
