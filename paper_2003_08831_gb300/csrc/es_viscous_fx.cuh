@@ -16,8 +16,22 @@ struct FxViscous {
 // z1 and z_v (z_k = nz_k 2^(ev - 62), |nz| < 2^62), iz1 = 1/z1 > 0 with z1 above an eighth of 2^e1.
 //   b_mk = theta_m,k - v_k theta_m,3, tau_mk = mu a (b_mk + b_km - 2/3 delta_mk tr b), a = 1/z1^2
 //   fV_m = (tau_m1, tau_m2, tau_m3, -kappa a^2/R theta_m,3 + sum_k tau_mk v_k)
-ES_HD void fx_viscous_flux(const fx t[3][4], const fx nz[3], double iz1, int e1, int ev, int ut, const FxViscous& V,
+// The gradients are brought to the top of their 62 bits first: along a line they are fractions of the largest that
+// the element's w could have at its thinnest weight, some 2^8 above what they are, and six bits are room below.
+ES_HD void fx_viscous_flux(const fx t0[3][4], const fx nz[3], double iz1, int e1, int ev, int ut, const FxViscous& V,
                            double f[3][4]) {
+  int top = 1;
+#pragma unroll
+  for (int m = 0; m < 3; ++m)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) top |= fx_hi(t0[m][c]) ^ (fx_hi(t0[m][c]) >> 31);
+  const int up = fx_clz(uint64_t(unsigned(top))) - 34;
+  fx t[3][4];
+#pragma unroll
+  for (int m = 0; m < 3; ++m)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) t[m][c] = t0[m][c] << up;
+  ut -= up;
   const int hi = fx_hi_word(iz1) >> 20, ei = hi - 1022;
   const fx ni = fx_from_positive(iz1, hi);  // 2^61 .. 2^62
   fx v[3];
