@@ -360,12 +360,13 @@ ES_HD int fx_unit(const FxScale& s, int v) {
 
 // Twice Q_ij = omega_i D_ij times the Ismail--Roe flux between two nodes, in units of 2^fx_unit
 // (a, b: z1, z_m, two other z_v, z5 as fractions of the block scales, 63 fractional bits; fa, fb:
-// z1 and z5 as float pairs; Q: Q_ij / 4 with 65, |Q_ij| < 0.7 for p = 2..5).  With S = a + b, 1/S1 = inv, g = 4 g5 = 1 - eps,
+// z1 and z5 as float pairs; Q: Q_ij / 4 with 65, |Q_ij| < 0.98 for p = 2..5).  With S = a + b, 1/S1 = inv, g = 4 g5 = 1 - eps,
 // f1 = 1 + del (see ec_flux):
 //   pq = Q S5/S1, M = g pq S_m, mass flux M S1, momentum M S_k (+ pq for k = m),
 //   energy u_m (g pq t + 2^(1-kt) pq), u_m = S_m/S1, t = C1x f1 + |S_v|^2/2 (scaled by 2^-kt).
 // Every factor Q multiplies once, so the pair enters both nodes' sums with opposite signs.
-// Bounds: 1/3 <= S1 < 1 (near: 0.49), so inv < 3 (2.05), pq < 0.57 (0.39), |u_m| < 3, t < 0.95.
+// Bounds: 1/3 <= S1 < 1 (near: 0.49), so inv < 3 (2.05), pq < 0.74 (0.5), |u_m| < 3 (2.05), t < 0.95 (0.88, with
+// 2^-kt <= 1/16 beside it, 0.82 with 1/8), so 4 y < 0.8 (8 y < 0.95) of 2^63.
 template <int TIER>
 ES_HD void fx_flux(const fx a[5], const FxPair fa[2], const fx b[5], const FxPair fb[2], fx Q, const FxScale& c,
                    fx g[5]) {

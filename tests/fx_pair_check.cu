@@ -2,6 +2,8 @@
 //   slow  gas slower than the velocities' other scales: mass and energy flux relative to themselves
 //   room  the room that fluxes beyond an element's scales are given
 //   near  the logarithmic-mean correction and the flux up to the limit of the near tier
+//   sums  sums along a line with the operators' own Q_ij, states at the corners of the range: a sum that leaves
+//         2^61 is seen, though it may wrap past 2^63
 //   metrics  rates of an element with anisotropic metrics, flow along the coarse direction
 #include <algorithm>
 #include <cmath>
@@ -252,6 +254,47 @@ int main(int argc, char** argv) {
         puts("");
       }
   }
+  if (!strcmp(argv[1], "sums"))
+    for (int p = 2; p <= 5; ++p) {
+      const Line l(p);
+      L largest = 0, q = 0;
+      int missed = 0, beyond = 0, out = 0, n = 0;
+      for (int i = 0; i <= p; ++i)
+        for (int j = 0; j <= p; ++j) q = std::max(q, fabsl(l.Q[i][j]));
+      for (double gam : {1.4, 5.0 / 3.0 + 1e-6, 1.1, 4.0})
+        for (int it = 0; it < 30000; ++it) {
+          // z1 and z5 at the ends of a factor 1.498 (near: 1.0098), from a power of two up or just below one
+          const Gas gas(gam);
+          const double f = it % 3 ? 1 / 1.498 : 1 / 1.0098, v = it % 2 ? 0.99999 : (it % 4 ? 1.99 : 3.99);
+          const double lo1 = it % 5 ? 1.0000001 : 1.9999, lo5 = it % 7 ? 1.9999 : 1.0000001;
+          double z[7][5];
+          __int128 r[6][5];
+          for (int i = 0; i < 7; ++i) {  // (node 7: elsewhere in the element, holds the scales)
+            z[i][0] = i == 6 ? lo1 : lo1 * (U(R) > 0 ? 1 : f);
+            z[i][4] = i == 6 ? lo5 : lo5 * (U(R) > 0 ? 1 : f);
+            for (int k = 1; k < 4; ++k) z[i][k] = v * (i == 6 ? 1 : (it % 11 ? (U(R) > 0 ? 1 : -1) : U(R)));
+          }
+          const FxScale t = scale(z, 7, gas);
+          if (t.tier == kFxSlow) {
+            ++out;
+            continue;
+          }
+          ++n;
+          line_sums(l, z, t, r);
+          for (int i = 0; i <= p; ++i)
+            for (int c = 0; c < 5; ++c)
+              for (int side = -1; side < 2; ++side) {  // with the largest face flux that is taken, or none
+                const __int128 e = r[i][c] + (i == 0 || i == p ? (__int128)side << (t.tier == kFxNear ? 61 : 60) : 0);
+                const fx w = fx(e);
+                const bool seen = ((fx_hi(w) + 0x20000000) & 0xc0000000) != 0;
+                largest = std::max(largest, fabsl((L)e));
+                const bool big = e >= ((__int128)1 << 61) || e < -((__int128)1 << 61);
+                beyond += big;
+                missed += big != seen;
+              }
+        }
+      printf("sums %d out %d beyond %d missed %d largest %.3Lf Q %.3Lf\n", p, out, beyond, missed, ldexpl(largest, -63), q);
+    }
   if (!strcmp(argv[1], "metrics"))
     for (int p = 2; p <= 5; ++p)
       for (double ratio : {1.0, 3.9, 7.9, 15.9, 16.5, 17.5, 33.0, 1e3}) {

@@ -10,6 +10,7 @@ Bounds.
   in the header), and the flux is no further from long double than the FP64 kernels' form of it, on average and
   at worst.
 * Metrics: where they are taken, the sums are no further off than the same sums in FP64.
+* Line sums: below 2^63 for the operators' own Q_ij with the largest face flux that is taken.
 """
 import os
 import shutil
@@ -60,6 +61,16 @@ def test_near_tier_to_its_limit(check):
         values = list(map(float, ln[5:13]))  # mean mass, energy; largest mass, energy: fixed point, FP64
         for fixed, double in zip(values[::2], values[1::2]):
             assert fixed <= double, ln
+
+
+def test_line_sums(check):
+    rows = check("sums")
+    assert len(rows) == 4
+    for ln in rows:
+        assert int(ln[3]) == 0 and int(ln[5]) > 0, ln
+        assert int(ln[7]) == 0, ln          # every sum beyond 2^61 is seen
+        assert float(ln[9]) < 1.0, ln       # none passes 2^63
+        assert float(ln[11]) < 0.98, ln
 
 
 def test_metrics(check):
