@@ -48,10 +48,21 @@ extern "C" {
                        (Section 4 pairs p = 4 with a fifth-order BSRK(8,5) whose coefficients
                        it does not print; es_set_tableau loads any explicit tableau) */
 
-#define ES_FP64 0  /* FP64, and 64-bit fixed point with per-element block exponents (58..63
-                      fractional bits) in the flux differencing where its error is no larger */
-#define ES_MIXED 1 /* FP32 fluxes/SATs/viscous terms; FP64 state, stage states,
-                      entropy-variable increments, entropy sums and gamma solve */
+#define ES_FP64 0  /* FP64 state, stage values and sums.  The parameter vector, the entropy-variable
+                      increments, flux differencing, interface fluxes (the Rusanov jump
+                      included, the matrix dissipation and diss^V in FP64), gradients, viscous
+                      fluxes and divergence and the gamma solve are formed in 64-bit fixed
+                      point (58..63 fractional bits of an element's, a node's or a pair's
+                      largest values) where that is no less accurate than FP64, and in FP64
+                      elsewhere: an element (a pair of face nodes) at rest or slower than about
+                      1e-9 of the sound speed or faster than Mach 3, or whose z1 = sqrt(rho/p) or
+                      z5 = sqrt(rho p) vary by more than a factor 1.5; meshes whose element
+                      sides differ by more than 16 (by up to 32 for some); increments of
+                      more than 2 % (the gamma solve: 1/16; gamma_gas below 17/16 or from
+                      3 on; roots outside 0.5..1.5). */
+#define ES_MIXED 1 /* FP32 fluxes/SATs/viscous terms; FP64 state and stage states;
+                      entropy-variable increments, entropy sums and gamma solve in FP64, the
+                      increments and the gamma solve as in ES_FP64 */
 #define ES_FP64X 2 /* fluxes/SATs/viscous terms in float-float arithmetic on the FP32 pipe
                       (hi + lo pairs of floats, ~2^-47 relative per operation, FP32 exponent
                       range), and so are the stage states, entropy-variable increments,
@@ -100,7 +111,9 @@ typedef struct {
                            width <= 4 2^-52 max(1, gamma).  In [0, 1); 0 selects 1e-8,
                            whose quadratic convergence leaves an error near 1e-16 gamma.
                            The float-float solves (ES_FP64X, ES_MIXED_FF) use at least
-                           2^-40 and stop at a bracket of width 2^-44 max(1, gamma). */
+                           2^-40 and stop at a bracket of width 2^-44 max(1, gamma); the
+                           fixed-point solves (ES_FP64) always go on to 2^-38, which leaves
+                           an error below 2^-53 gamma. */
 } es_config;
 
 /* Mesh, LGL/SBP tables (Section 3.1: diagonal-norm SBP on LGL nodes) and
@@ -275,7 +288,9 @@ int es_autotune(es_ctx* ctx, const double* q, void* stream);
  * kernel from the neighbours' parameter vectors, so the face-flux kernel and its
  * round trip through memory drop out (available for FP32 fluxes, ES_MIXED and
  * ES_MIXED_FF, on periodic Euler meshes; each face's flux is then evaluated by both
- * of its elements).  Every variant gives bit-identical results; 0 is the default.  es_set_volume_variant returns
+ * of its elements).  Every variant gives bit-identical results; 0 is the default.
+ * ES_FP64 meshes (and batch groups) of at most 600 elements have one tile of their own: the
+ * variant is kept but has no effect, and es_autotune has nothing to choose.  es_set_volume_variant returns
  * ES_ERR_INVALID for a variant outside 0..5 or a fused one the context cannot use;
  * es_autotune picks among all usable variants. */
 int es_volume_variant(const es_ctx* ctx);

@@ -554,7 +554,8 @@ int ensure_stage_buffers(Group& g, int s) {
 }
 
 // Allocates a group for the instances `insts` (same degree and physics).
-int group_init(Group& g, const es_config* insts, int n, int stages, bool own_state) {
+int group_init(Group& g, const es_config* insts, int n, const Engine& E, bool own_state) {
+  const int stages = E.tab.s;
   const es_config& C = insts[0];
   g.cfg = C;
   g.P1 = C.p + 1;
@@ -563,6 +564,7 @@ int group_init(Group& g, const es_config* insts, int n, int stages, bool own_sta
   g.tf = (C.precision == ES_MIXED || C.precision == ES_MIXED_FF) ? 4 : 8;  // bytes per flux value (float-float: 8)
   g.ffx = C.precision == ES_FP64X;
   build_params(C, &g.P);
+  g.P.sms = E.sm_count;
   long long K = 0;
   g.geom.resize(n);
   for (int i = 0; i < n; ++i) {
@@ -870,6 +872,8 @@ int status_read(Engine& E, cudaStream_t st) {
 
 // Times each volume tile on the group's current state (one stage's RHS) and keeps the fastest.
 int autotune_group(Engine& E, Group& g, const double* q, cudaStream_t st) {
+  // (small FP64 groups have one tile)
+  if (g.tf == 8 && !g.ffx && g.K <= kSmallMesh) return cuda_check(cudaStreamSynchronize(st));
   cudaEvent_t a, b;
   if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return ES_ERR_CUDA;
   float best = 1e30f;
@@ -937,7 +941,7 @@ int es_create(const es_config* cfg, es_ctx** out) {
   es_ctx* c = new (std::nothrow) es_ctx();
   if (!c) return ES_ERR_NOMEM;
   int rc = engine_init(c->eng, C);
-  if (rc == ES_OK) rc = group_init(c->g, &C, 1, c->eng.tab.s, false);
+  if (rc == ES_OK) rc = group_init(c->g, &C, 1, c->eng, false);
   if (rc != ES_OK) {
     group_free(c->g);
     engine_free(c->eng);
@@ -1269,7 +1273,7 @@ int es_batch_create(const es_config* cfgs, int count, es_batch** out) {
     if (insts.empty()) continue;
     b->groups.emplace_back();
     Group& g = b->groups.back();
-    rc = group_init(g, insts.data(), (int)insts.size(), b->eng.tab.s, true);
+    rc = group_init(g, insts.data(), (int)insts.size(), b->eng, true);
     g.inst_ids = ids;
     for (size_t j = 0; j < ids.size(); ++j) b->where[ids[j]] = {(int)b->groups.size() - 1, (int)j};
   }

@@ -91,6 +91,7 @@ struct FxParams : Params {
   long long fxI;                   // 1/(gam - 1) = fxI 2^(fxEi - 62), 2^61 <= fxI < 2^62
   int fxKt, fxKw, fxEg, fxEi;
   int fxIso;                       // fx_metrics_close of every instance
+  int sms;                         // SMs of the device (host side: block sizes)
 };
 
 template <typename T> __device__ __forceinline__ const FluxConst<T>& flux_const(const Params& P);

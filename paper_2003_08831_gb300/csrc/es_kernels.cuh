@@ -1930,13 +1930,10 @@ __global__ void k_estimate(Params P, const double* __restrict__ q, const double*
 // ---------------------------------------------------------------------------
 // launchers
 
-// Meshes that leave SMs idle: a tile of one element and all three directions takes 12 to 21 us up to
-// 512 elements where the larger tiles take 21 to 39 (p = 2, 3, 5); at 1000 elements they meet for p = 3.
-constexpr int kSmallMesh = 600;
 // Threads per block of the kernels that work node by node: blocks of 64 while blocks of 256 would
-// not give every SM one (152 SMs).
-inline int node_block(int& grid) {
-  if (grid > 152) return 256;
+// not give every SM one.
+inline int node_block(const FxParams& P, int& grid) {
+  if (grid > P.sms) return 256;
   grid *= 4;
   return 64;
 }
@@ -1944,7 +1941,7 @@ inline int node_block(int& grid) {
 template <typename TF, bool FP64, bool BC>
 void prep_launch(const FxParams& P, const StagePrep& sp, TF* a, int* status, cudaStream_t st, int grid,
                  const std::conditional_t<BC, BcEval, int>& bc) {
-  const int nb = node_block(grid);
+  const int nb = node_block(P, grid);
   if (BC) ++grid;
   // Small meshes wait for the chain of a node's operations: parameter vector and increment by different
   // threads (isentropic vortex 4^3 p = 3: 5.2 -> 4.8 us per launch).
@@ -1984,7 +1981,7 @@ void Launcher<P1, TF>::prep(const FxParams& P, const StagePrep& sp, void* aux, i
 
 template <int P1, typename TF>
 void Launcher<P1, TF>::face(const FxParams& P, const void* aux, void* F, void* FL, cudaStream_t st, int grid) {
-  const int nb = node_block(grid);
+  const int nb = node_block(P, grid);
   const TF* a = static_cast<const TF*>(aux);
   TF *f = static_cast<TF*>(F), *fl = static_cast<TF*>(FL);
   if constexpr (std::is_same<TF, double>::value) {
@@ -2125,7 +2122,7 @@ void Launcher<P1, TF>::relax(const FxParams& P, const StageRelax& sr, cudaStream
   const bool fp64 = sr.u_new || std::is_same<TF, double>::value || (std::is_same<TF, float>::value && !P.ff_est);
   // (one warp per block while four would leave SMs idle)
   const int epw = fp64 ? RelaxGroup<P1>::EPW : RelaxGroup<P1, true>::EPW;
-  const int warps = P.K < 4 * epw * 152 ? 1 : 4;
+  const int warps = P.K < 4 * epw * P.sms ? 1 : 4;
   const int need = (P.K + warps * epw - 1) / (warps * epw);
   const int g = std::min(grid * 4 / warps, need);
   if (fp64 && sr.u_new) k_relax<P1, true><<<g, 32 * warps, 0, st>>>(P, sr);

@@ -96,6 +96,10 @@ constexpr int kGlobalRelaxIterations = 8;
 // interface fluxes formed in the volume kernel (FP32 fluxes on periodic Euler groups)
 constexpr int kVolumeVariants = 3;
 constexpr int kStageVariants = 2 * kVolumeVariants;
+// FP64 meshes that leave SMs idle have a tile of their own, whatever variant is asked for: one element per
+// block and all three directions take 12 to 21 us up to 512 elements where the larger tiles take 21 to 39
+// (p = 2, 3, 5); at 1000 elements they meet for p = 3.
+constexpr int kSmallMesh = 600;
 
 // Dirichlet-penalty boundary data of a context
 struct BcSpec {

@@ -135,6 +135,7 @@ extern "C" int es_rhs_noalloc(const es_config* cfg, const double* q, double* dqd
   sv.kout64 = dqdt;
   sv.E = E_elem;
   const int sms = g_sm_count[dev];
+  P.sms = sms;
   const bool ns = cfg->mu > 0.0;
   rc = dispatch_p1(P1, fp64, [&](auto L) {
     using Lc = decltype(L);

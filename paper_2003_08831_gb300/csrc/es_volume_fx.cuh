@@ -260,10 +260,10 @@ __device__ __forceinline__ int volume_line_fx(const FxParams& P, const FxScale& 
 }
 
 // Tiles (elements per CTA, threads) and register bounds, measured on GB300 (one right-hand side,
-// 2 M nodes, us): the kernel waits on the latency of its dependent integer products, so few
-// registers pay until they spill into the sums.  p = 2: 199 at 16 x 160 and 96 registers (32 x 288:
-// 222); p = 3: 211 at 4 x 64 and 168 (128: 213, 96: 235; 8 x 128: 229); p = 4: 283 at 1 x 32 and
-// 128 (5 x 128: 286); p = 5: 328 at 2 x 96 and 168 (4 x 160: 353, 1 x 64: 409).
+// tiles 0, 1 and 2, us): the kernel waits on the latency of its dependent integer products, so few
+// registers pay until they spill into the sums.  Taylor--Green 48^3 p = 2: 297, 319, 318; 40^3 p = 3: 447, 416,
+// 421; 32^3 p = 4: 565, 676, 668 (the second at 128 registers 698); 24^3 p = 5: 620, 633, 800; Navier--Stokes 24^3
+// p = 4: 390, 471, 459 (the second at 128 registers 510).
 // Variant 3 is for meshes of few elements, whatever tile is asked for (the bits are the same): one
 // element per CTA and a thread for every line of its three directions.
 constexpr int kVolFxSmall = 3;
