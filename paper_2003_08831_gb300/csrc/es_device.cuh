@@ -95,7 +95,6 @@ struct FxParams : Params {
 };
 
 template <typename T> __device__ __forceinline__ const FluxConst<T>& flux_const(const Params& P);
-template <> __device__ __forceinline__ const FluxConst<double>& flux_const<double>(const Params& P) { return P.Cd; }
 template <> __device__ __forceinline__ const FluxConst<float>& flux_const<float>(const Params& P) { return P.Cf; }
 template <> __device__ __forceinline__ const FluxConst<ff>& flux_const<ff>(const Params& P) { return P.Cff; }
 
@@ -150,10 +149,6 @@ __device__ __forceinline__ double mass_weight(const Params& P, double J, int n) 
 
 // operator entries in the flux precision T (float-float: the split tables)
 template <typename T> struct Tab;
-template <> struct Tab<double> {
-  static __device__ __forceinline__ double D(const Params& P, int i) { return P.D[i]; }
-  static __device__ __forceinline__ double D2(const Params& P, int i) { return P.D2[i]; }
-};
 template <> struct Tab<float> {
   static __device__ __forceinline__ float D(const Params& P, int i) { return P.Dff[0][i]; }
   static __device__ __forceinline__ float D2(const Params& P, int i) { return P.D2ff[0][i]; }
@@ -164,8 +159,7 @@ template <> struct Tab<ff> {
 };
 
 // acc += a b in the flux precision (the float-float form keeps the product and
-// sum errors, see es_ff.cuh; FP64/FP32 use one fma, as contraction would)
-__device__ __forceinline__ void fma_acc(double& acc, double a, double b) { acc = fma(a, b, acc); }
+// sum errors, see es_ff.cuh; FP32 one fma, as contraction would)
 __device__ __forceinline__ void fma_acc(float& acc, float a, float b) { acc = fmaf(a, b, acc); }
 __device__ __forceinline__ void fma_acc(ff& acc, ff a, ff b) { ff_fma_acc(acc, a, b); }
 

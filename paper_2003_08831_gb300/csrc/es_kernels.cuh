@@ -298,7 +298,6 @@ __device__ __forceinline__ bool param_vector_ff(const ff y[5], const FluxConst<f
 }
 
 // FP64 value of a flux-precision value (float: the bits placed on the integer pipe)
-__device__ __forceinline__ double to_f64(double x) { return x; }
 __device__ __forceinline__ double to_f64(float x) { return f32_to_f64_bits(x); }
 __device__ __forceinline__ double to_f64(ff x) { return double(x); }
 
@@ -1079,9 +1078,9 @@ __device__ __forceinline__ void volume_body(const Params& P, const StageVol& sv,
   // node phase: write k_i (or, in the last stage, d = sum_j c_j k_j + c_self k_i), element sums
   const bool wantE = sv.E != nullptr;
   const bool wantA = sv.dw != nullptr;
-  // d and the element sums in FP64 (FP64 mode; mixed mode with FP64 estimates), else
+  // d and the element sums in FP64 (mixed mode with FP64 estimates), else
   // in float-float joined to FP64 once
-  const bool fp64_sums = std::is_same<TF, double>::value || (std::is_same<TF, float>::value && !P.ff_est);
+  const bool fp64_sums = std::is_same<TF, float>::value && !P.ff_est;
   for (int t = threadIdx.x; t < nn; t += blockDim.x) {
     const long long g = (long long)e0 * Np + t;
     const int n = t % Np;
