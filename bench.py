@@ -17,7 +17,6 @@ problems, no data-path collective: weak scaling); rank 0 prints one JSON line.
 the same workload (rank 0 only).
 """
 import argparse
-import hashlib
 import json
 import math
 import os
@@ -95,28 +94,6 @@ def volume_flops_per_element(p, ns=False, with_A=False):
 FACE_FLOPS_PER_FACE_NODE = 56 + 55
 PREP_FLOPS_Z, PREP_FLOPS_PER_STAGE, PREP_FLOPS_PENDING, PREP_FLOPS_DW = 22, 10, 10, 122
 RELAX_FLOPS_SETUP, RELAX_FLOPS_CUBIC, RELAX_FLOPS_EVAL = 65, 20, 75
-
-
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the k_volume launches of one
-# step of the default workload (stages 1, 2, 3; FP64, tile variant 1), from the ncu capture
-# summarised in profiles/; the roofline reports their mean, per launch like `achieved`.
-# It is reported only while the kernel sources hash to the value the capture was taken with.
-VOLUME_TRAFFIC = {"source_sha1": "9ead7ce83383f973f27e285f991389a131516fd2",
-                  "bytes_per_stage": [148340480 + 48874752, 232487680 + 55985664, 400438528 + 65617408]}
-
-
-def kernel_source_sha1():
-    h = hashlib.sha1()
-    for f in ("es_kernels.cuh", "es_device.cuh", "es_ff.cuh"):
-        with open(os.path.join(ROOT, "paper_2003_08831_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest()
-
-
-def fp_peak_tflops(precision, sm_mhz):
-    """ALU peak from unit counts x clock: 152 SMs, FP64 2 DFMA/clk/SM, FP32 128 FFMA/clk/SM."""
-    per_clk = 4.0 if precision == 0 else 256.0
-    return 152 * per_clk * sm_mhz * 1e6 / 1e12
 
 
 def hbm_peak_gbs():
@@ -231,6 +208,17 @@ def kernel_rooflines(p, n_el, precision, prof, peaks, ns=False):
         out[k] = {"avg_launch_ms": ms / n, "flops": {a: v for a, v in fl.items()}, "bytes": by,
                   "frac_fp64": t64 / t, "frac_fp32": t32 / t, "frac_hbm": tb / t,
                   "bound": bound, "frac": troof / t}
+    return out
+
+
+def fixed_point_rooflines(kr):
+    """kernel_rooflines of the FP64 mode, whose kernels do most of that work on the integer pipe: HBM is
+    the roofline, and the FP64 pipe's time for the same operations over the launch time is only a
+    comparison (fp64_equivalent, above one where the integer pipe is ahead)."""
+    out = {}
+    for k, v in kr.items():
+        w = {a: b for a, b in v.items() if a not in ("frac_fp64", "frac_fp32")}
+        out[k] = dict(w, bound="hbm", frac=v["frac_hbm"], fp64_equivalent=v["frac_fp64"])
     return out
 
 
@@ -695,6 +683,8 @@ def main():
     ap.add_argument("--workload", default=MAIN, choices=sorted(WORKLOADS))
     ap.add_argument("--no-forms", action="store_true", help="skip the extra precision/physics forms")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU oracle baseline")
+    ap.add_argument("--full", default=os.path.join(ROOT, "bench_full.json"),
+                    help="file for the whole record (every form, per-kernel times and rooflines)")
     ap.add_argument("--quick", action="store_true",
                     help="timed region only (no kernel-event pass, e2e, forms or CPU baseline): for profilers")
     args = ap.parse_args()
@@ -709,20 +699,33 @@ def main():
 
 
 def compact(form):
-    """The few numbers of a form that the end of the JSON line repeats."""
-    out = {"value": form["value"], "ms_per_step": form["ms_per_step"]}
+    """The few numbers of a form that the printed line holds."""
+    out = {"value": float("%.4g" % form["value"])}
     kr = form.get("kernel_roofline") or {}
     if "volume" in kr:
-        out["volume_frac"] = round(kr["volume"]["frac"], 3)
-        out["volume_bound"] = kr["volume"]["bound"]
+        out["volume_bound"] = [kr["volume"]["bound"], round(kr["volume"]["frac"], 3)]
     if "speedup_vs_fp64_same_physics" in form:
         out["speedup_vs_fp64"] = round(form["speedup_vs_fp64_same_physics"], 3)
     if "error_vs_fp64" in form:
-        out["rel_l2_vs_fp64"] = form["error_vs_fp64"]["rel_l2"]
+        out["rel_l2_vs_fp64"] = float("%.2g" % form["error_vs_fp64"]["rel_l2"])
     if "degree_mix" in form:
-        out["predicted_from_degree_mix"] = form["degree_mix"]["predicted_from_degree_mix"]
-        out["measured_over_predicted"] = round(form["degree_mix"]["measured_over_predicted"], 3)
+        out["over_predicted"] = round(form["degree_mix"]["measured_over_predicted"], 3)
     return out
+
+
+def printed(out):
+    """The line on stdout: the headline and what belongs to it, short enough to be kept whole by a log
+    that holds only the end of the output; the file args.full has the rest."""
+    keep = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks", "e2e")
+    line = {k: out[k] for k in keep}
+    vol = out["kernel_roofline"]["volume"]
+    line["roofline"] = {"kernel": "k_volume", "bound": vol["bound"], "frac": round(vol["frac"], 3)}
+    if "cpu_baseline" in out:
+        line["cpu_baseline"] = {k: out["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    if "short" in out:
+        line["forms"] = out["short"]
+    return line
 
 
 def run_full(args, rank, world, local_rank):
@@ -760,15 +763,10 @@ def run_full(args, rank, world, local_rank):
     p = wl["p"]
     K = wl["n"] ** 3
     ns = wl["mu"] > 0
-    # average over the 3 stages: the A term is accumulated in stages 2 and 3
-    fl = K * (volume_flops_per_element(p, ns, False) + 2 * volume_flops_per_element(p, ns, True)) / 3.0
-    vol_ms, vol_n = prof["volume"]
-    avg_ms = vol_ms / max(vol_n, 1)
-    achieved = fl / (avg_ms * 1e-3) / 1e12
-    sm_mhz = clocks["sm_mhz"] if clocks else 2070.0
-    peak = fp_peak_tflops(wl["precision"], sm_mhz)
-    peak_meas = peaks["fp64_tflops"] if wl["precision"] == 0 else peaks["fp32_tflops"]
     tot = sum(v[0] for v in prof.values())
+    rooflines = kernel_rooflines(p, K, wl["precision"], prof, peaks, ns)
+    if wl["precision"] == 0:
+        rooflines = fixed_point_rooflines(rooflines)
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
@@ -777,21 +775,8 @@ def run_full(args, rank, world, local_rank):
         "config": workload_config(args.workload),
         "dt": res["dt"], "gamma_range": [res["gamma_min"], res["gamma_max"]],
         "gpu_launches": int(res["launches"]),
-        "roofline": {"bound": "alu", "kernel": "k_volume (flux differencing + SATs)",
-                     "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                     "traffic": (sum(VOLUME_TRAFFIC["bytes_per_stage"]) / 3.0
-                                 if VOLUME_TRAFFIC["source_sha1"] == kernel_source_sha1() and wl is WORKLOADS[MAIN]
-                                 else None),
-                     "traffic_unit": "bytes per launch, mean of the step's three launches (ncu, same kernel "
-                                     "sources)",
-                     "peak_source": "%s ALU peak from unit counts x median SM clock (%.0f MHz): 152 SMs x %s"
-                                    % ("FP64" if wl["precision"] == 0 else "FP32", sm_mhz,
-                                       "2 DFMA/clk" if wl["precision"] == 0 else "128 FFMA/clk"),
-                     "peak_measured": peak_meas, "frac_of_measured": achieved / peak_meas,
-                     "peak_measured_source": "FMA-chain throughput in this run (es_fma_peak)",
-                     "flops_per_launch": fl, "avg_launch_ms": avg_ms},
         "kernel_share": {k: round(v[0] / tot, 4) for k, v in prof.items() if v[1] > 0},
-        "kernel_roofline": kernel_rooflines(p, K, wl["precision"], prof, peaks, ns),
+        "kernel_roofline": rooflines,
         "clocks": clocks,
         "peaks_measured": dict(peaks, hbm_gbs=hbm_peak_gbs()[0], hbm_source=hbm_peak_gbs()[1]),
     }
@@ -814,12 +799,12 @@ def run_full(args, rank, world, local_rank):
             r2["solver"].close()
             t2 = sum(v[0] for v in p2.values())
             err = error_vs_fp64(w2) if w2["precision"] != 0 else None
+            roof2 = kernel_rooflines(w2["p"], w2["n"] ** 3, w2["precision"], p2, peaks, w2["mu"] > 0)
             forms[name] = {"value": r2["nodes"] * STAGES * steps2 / (r2["ms"] / 1e3),
                            "ms_per_step": r2["ms"] / steps2, "steps": steps2,
                            "gamma_range": [r2["gamma_min"], r2["gamma_max"]], "launches": int(r2["launches"]),
                            "kernel_share": {k: round(v[0] / t2, 4) for k, v in p2.items() if v[1] > 0},
-                           "kernel_roofline": kernel_rooflines(w2["p"], w2["n"] ** 3, w2["precision"], p2, peaks,
-                                                               w2["mu"] > 0),
+                           "kernel_roofline": roof2 if w2["precision"] else fixed_point_rooflines(roof2),
                            "speedup_vs_fp64_same_physics": None}
             if err is not None:
                 forms[name]["error_vs_fp64"] = err
@@ -851,19 +836,16 @@ def run_full(args, rank, world, local_rank):
                 del forms[k]["speedup_vs_fp64_same_physics"]
         out["forms"] = forms
         # the FP64 vs mixed pair on the largest single-instance workload (Navier--Stokes TGV,
-        # 32^3, p = 4) and the other forms, repeated compactly at the end of the line
-        out["ns_fp64"] = compact(forms["tgv_ns_re1600_p4_32^3_fp64"])
-        out["ns_mixed"] = compact(forms["tgv_ns_re1600_p4_32^3_mixed_noise"])
-        out["ns_mixed_ff"] = compact(forms["tgv_ns_re1600_p4_32^3_mixed_ff_noise"])
-        out["ns_fp64x"] = compact(forms["tgv_ns_re1600_p4_32^3_fp64x"])
-        out["euler_mixed"] = compact(forms["tgv_euler_p3_32^3_mixed"])
-        out["euler_mixed_ff"] = compact(forms["tgv_euler_p3_32^3_mixed_ff"])
-        out["euler_fp64x"] = compact(forms["tgv_euler_p3_32^3_fp64x"])
-        out["batch_fp64"] = compact(forms["batched_vortex_256_fp64"])
-        out["batch_mixed_ff"] = compact(forms["batched_vortex_256_mixed_ff"])
-    out["headline_volume_frac"] = {"of_unit_count_peak": round(achieved / peak, 3),
-                                   "of_measured_fma_peak": round(achieved / peak_meas, 3)}
-    print(json.dumps(out), flush=True)
+        # 32^3, p = 4) and the other forms
+        short = {"ns_fp64": "tgv_ns_re1600_p4_32^3_fp64", "ns_mixed": "tgv_ns_re1600_p4_32^3_mixed_noise",
+                 "ns_mixed_ff": "tgv_ns_re1600_p4_32^3_mixed_ff_noise", "ns_fp64x": "tgv_ns_re1600_p4_32^3_fp64x",
+                 "euler_mixed": "tgv_euler_p3_32^3_mixed", "euler_mixed_ff": "tgv_euler_p3_32^3_mixed_ff",
+                 "euler_fp64x": "tgv_euler_p3_32^3_fp64x", "batch_fp64": "batched_vortex_256_fp64",
+                 "batch_mixed_ff": "batched_vortex_256_mixed_ff"}
+        out["short"] = {k: compact(forms[v]) for k, v in short.items()}
+    with open(args.full, "w") as f:
+        json.dump(out, f, indent=1)
+    print(json.dumps(printed(out)), flush=True)
     if dist is not None:
         dist.barrier()
     return 0
