@@ -212,13 +212,15 @@ def kernel_rooflines(p, n_el, precision, prof, peaks, ns=False):
 
 
 def fixed_point_rooflines(kr):
-    """kernel_rooflines of the FP64 mode, whose kernels do most of that work on the integer pipe: HBM is
-    the roofline, and the FP64 pipe's time for the same operations over the launch time is only a
-    comparison (fp64_equivalent, above one where the integer pipe is ahead)."""
+    """kernel_rooflines of the modes that do their FP64 work (ES_FP64: most of it, ES_MIXED: the increments
+    and the gamma solve) on the integer pipe: HBM or the FP32 pipe is the roofline, and the FP64 pipe's time for
+    the same operations over the launch time is only a comparison (fp64_equivalent, above one where the
+    integer pipe is ahead)."""
     out = {}
     for k, v in kr.items():
-        w = {a: b for a, b in v.items() if a not in ("frac_fp64", "frac_fp32")}
-        out[k] = dict(w, bound="hbm", frac=v["frac_hbm"], fp64_equivalent=v["frac_fp64"])
+        w = {a: b for a, b in v.items() if a != "frac_fp64"}
+        bound = "fp32" if v["frac_fp32"] > v["frac_hbm"] else "hbm"
+        out[k] = dict(w, bound=bound, frac=v["frac_" + bound], fp64_equivalent=v["frac_fp64"])
     return out
 
 
@@ -765,7 +767,7 @@ def run_full(args, rank, world, local_rank):
     ns = wl["mu"] > 0
     tot = sum(v[0] for v in prof.values())
     rooflines = kernel_rooflines(p, K, wl["precision"], prof, peaks, ns)
-    if wl["precision"] == 0:
+    if wl["precision"] in (0, 1):
         rooflines = fixed_point_rooflines(rooflines)
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -804,7 +806,7 @@ def run_full(args, rank, world, local_rank):
                            "ms_per_step": r2["ms"] / steps2, "steps": steps2,
                            "gamma_range": [r2["gamma_min"], r2["gamma_max"]], "launches": int(r2["launches"]),
                            "kernel_share": {k: round(v[0] / t2, 4) for k, v in p2.items() if v[1] > 0},
-                           "kernel_roofline": roof2 if w2["precision"] else fixed_point_rooflines(roof2),
+                           "kernel_roofline": fixed_point_rooflines(roof2) if w2["precision"] in (0, 1) else roof2,
                            "speedup_vs_fp64_same_physics": None}
             if err is not None:
                 forms[name]["error_vs_fp64"] = err
