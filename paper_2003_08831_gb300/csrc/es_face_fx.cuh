@@ -2,7 +2,7 @@
 // of face nodes in the scales of that pair, and the Rusanov dissipation lambda/2 [[q]] from the
 // same fractions.  An FP64 face node takes 42 + 44 FP64 instructions, each the time of ~76 of one
 // scheduler's; this takes about 900 integer and FP32 ones.  Taylor--Green 32^3 p = 3: k_face
-// 244 -> 123 us per launch.
+// 244 -> 101 us per launch, with the launch shape of k_face_fp64.
 #pragma once
 #include "es_fx.cuh"
 

@@ -9,7 +9,7 @@
 // units, so a node's flux carries 2^-56 of (its element's w) (2/h)/omega, against FP64's 2^-53 for
 // every one of the sum's terms.
 //
-// Per launch: Navier--Stokes p = 4 32^3 1167 -> 510 us, viscous shock p = 3 25^3 267 -> 124 us
+// Per launch: Navier--Stokes p = 4 32^3 1167 -> 525 us, viscous shock p = 3 25^3 267 -> 127 us
 // (80, 96 and 168 registers per thread: within 3 % of 128).
 #pragma once
 #include "es_viscous_fx.cuh"

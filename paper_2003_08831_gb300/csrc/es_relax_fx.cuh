@@ -15,7 +15,7 @@
 //
 // An FP64 solve took about 60 FP64 instructions per node and 90 more per Newton step, each the
 // time of 76 scheduler slots (es_fx.cuh); this takes about 1200 slots in all.  k_relax per launch:
-// Taylor--Green 32^3 p = 3 471 -> 136 us, p = 4 1042 -> 285 us; 11 x 9 x 13 p = 5 90 -> 37 us; entry
+// Taylor--Green 32^3 p = 3 471 -> 140 us, p = 4 1042 -> 285 us; 11 x 9 x 13 p = 5 90 -> 39 us; entry
 // point with u_new, 17 x 13 x 19 p = 2 (two FP64 logarithms per node remain) 75 -> 43 us.  Against long
 // double the root is 3 to 10 times closer than FP64's (tests/test_fx_relax.py).
 #pragma once

@@ -4,9 +4,9 @@
 // Bound: the FP64 form spent 84 % of its time on the FP64 pipe (52 FP64 instructions per pair of
 // nodes, ~76 scheduler slots each).  A pair now takes about 230 integer and FP32 instructions, half
 // of them on the half-rate ALU pipe, which sets the time.  Taylor--Green 32^3 p = 3, one stage's
-// launch (mean of a step's three): 1089 us -> 258 us; p = 5, 11 x 9 x 13: 363 us -> 93 us.
-// Accuracy against long double (right-hand side, per variable): no larger error than FP64's in any
-// variable, half of it in the momentum; element sums equal to two digits.
+// launch (mean of a step's three): 1089 us -> 254 us; p = 5, 11 x 9 x 13: 363 us -> 100 us.
+// Accuracy against long double (right-hand side, 149 states, per variable): 0.29 of the FP64 form's
+// error in the median, 1.06 at most; element sums equal to two digits.
 #pragma once
 #include "es_fx.cuh"
 
@@ -353,8 +353,9 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * REGS)) k_volume_fx
     }
     // Where the viscous fluxes may not fit: looked at before any pair is formed, and the room they need
     // given at once (an element that does not fit all the same is found below).
-    // Viscous shock 25^3 p = 3 693 -> 540 us per launch; looked at without the estimate before it, Navier--
-    // Stokes p = 4 takes 941 us (930 with, 924 with neither).
+    // Viscous shock 25^3 p = 3 693 -> 540 us per launch (576 with the room that every element is given now,
+    // three bits or what it needs); looked at without the estimate before it, Navier--Stokes p = 4 takes
+    // 941 us (930 with, 924 with neither).
     if constexpr (NS) {
       if (__syncthreads_or(viscous)) {
 #pragma unroll 1
